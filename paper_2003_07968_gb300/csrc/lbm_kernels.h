@@ -3,6 +3,7 @@
 #include <cuda.h>
 
 #include "lbm_device.cuh"
+#include "lbm_rows_plan.h"
 
 namespace pplbm {
 
@@ -71,5 +72,11 @@ cudaError_t launch_fused_tma(int f16, int mrt, int eos, int tx, int ty, const St
                              const CUtensorMap* map, const LatDev* lat0, int grid,
                              cudaStream_t st);
 int occupancy_fused_tma(int f16, int mrt, int eos, int tx, int ty, bool with_map, bool single);
+// Many steps in one cooperative launch over a resident plan's tiles
+// (float-float EOS; lbm_rows.cuh): lat0 as in launch_fused_tma.  All blocks
+// must be resident together: grid at most SMs x resident_blocks_per_sm.
+cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
+                            size_t smem, cudaStream_t st);
+int resident_blocks_per_sm(int f16, int mrt, bool single, size_t smem);
 
 }  // namespace pplbm

@@ -1,0 +1,23 @@
+// lbm_rows.cu -- host side of the row kernels: dispatch to the instance units
+// (lbm_rows_{f32,f16}.cu; the kernels are in lbm_rows.cuh).
+#include "lbm_kernels.h"
+
+namespace pplbm {
+
+cudaError_t resident_f32(int, const ResArgs*, const LatDev*, int, size_t, cudaStream_t, int*);
+cudaError_t resident_f16(int, const ResArgs*, const LatDev*, int, size_t, cudaStream_t, int*);
+
+cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
+                            size_t smem, cudaStream_t st) {
+    return (f16 ? resident_f16 : resident_f32)(mrt, &m, lat0, grid, smem, st, nullptr);
+}
+
+int resident_blocks_per_sm(int f16, int mrt, bool single, size_t smem) {
+    int occ = 0;
+    const LatDev lat{};
+    const cudaError_t e = (f16 ? resident_f16 : resident_f32)(mrt, nullptr, single ? &lat : nullptr,
+                                                             0, smem, nullptr, &occ);
+    return e == cudaSuccess ? occ : 0;
+}
+
+}  // namespace pplbm

@@ -1,0 +1,11 @@
+// lbm_rows_f32.cu -- instances of the row kernels: FP32 storage.
+#include "lbm_rows.cuh"
+
+namespace pplbm {
+
+cudaError_t resident_f32(int mrt, const ResArgs* m, const LatDev* lat0, int grid, size_t smem,
+                         cudaStream_t st, int* occ) {
+    return resident_any<StoreF32>(mrt, m, lat0, grid, smem, st, occ);
+}
+
+}  // namespace pplbm

@@ -1,0 +1,130 @@
+// lbm_rows_plan.h -- host side of the row kernels (lbm_rows.cuh): how lattices
+// are cut into strips of columns and bands of rows.
+#pragma once
+#include <algorithm>
+#include <vector>
+
+#include "lbm_device.cuh"
+
+namespace pplbm {
+
+constexpr int kRowCols = 60;  // columns a warp advances at most (it holds 64)
+
+// Column c of boundary k of n strips over nx columns: even, at most kRowCols
+// apart, as equal as that allows.
+inline int strip_edge(int nx, int n, int k) {
+    const int pairs = (nx + 1) / 2;
+    return std::min(nx, 2 * (int)(((int64_t)pairs * k + n - 1) / n));
+}
+inline int strip_count(int nx) { return (nx + kRowCols - 1) / kRowCols; }
+inline int band_edge(int ny, int n, int k) { return (int)((int64_t)ny * k / n); }
+
+// ---- resident lattices: one tile a block, kept in shared memory for many steps
+constexpr int kResWarps = 8;            // warps of a block, one row each at a time
+constexpr int kResSmem = 113 * 1024;    // shared memory of a block (two on an SM)
+constexpr int kResRows = 96;            // rows of a tile at most
+constexpr int kResMail = 1088;          // packets of a mailbox slot at most
+constexpr int kResBlocks = 480;         // blocks of a launch at most
+
+// packets of a tile's halo (three values each; see k_resident)
+constexpr int res_packets(int rows, int wd) { return 20 * ((wd + 2) / 3 + (rows + 2) / 3) + 40; }
+static_assert(res_packets(kResRows, kRowCols) <= kResMail, "a tile's halo fits its mailbox");
+static_assert((int64_t)kResBlocks * 2 * kResMail < 1 << 20, "a packet's place takes 20 bits");
+// shared memory of a tile: psi, packet table, lattice constants, the box (and
+// the elements a line's last packet may read past it)
+inline size_t res_smem(int rows, int wd, int es) {
+    return (size_t)(rows + 2) * 256 + (size_t)res_packets(rows, wd) * 8 + sizeof(LatDev) +
+           (size_t)9 * (rows + 4) * 64 * es + 256 * es;
+}
+// rows of the tallest tile that fits
+inline int res_rows(int es) {
+    int r = 2;
+    while (r < kResRows && res_smem(r + 1, kRowCols, es) <= (size_t)kResSmem &&
+           9 * (r + 5) * 64 <= 65536)
+        ++r;
+    return r;
+}
+
+struct ResTile {
+    int32_t lattice, x0, wd, y0, rows;
+    int32_t nbr[8];  // tiles above left, above, above right, left, right, below left, below, below right
+    int32_t wd_w, wd_e;  // widths of the left and right neighbours
+    int32_t gr_n, gr_s;  // (rows + 2) / 3 of the tiles above and below
+};
+struct ResArgs {
+    StepArgs a;
+    const ResTile* tiles;
+    uint4* mail;      // [tile][2][slot]
+    uint32_t* epoch;  // per tile: steps so far (all equal between launches)
+    int slot;         // packets of a mailbox slot
+    int nsteps;
+};
+
+// Bands of a lattice of ny rows when tiles of about `rows` rows are aimed at.
+inline int res_bands(int ny, int rows) { return std::max(1, std::min((ny + rows - 1) / rows, ny / 2)); }
+
+struct ResPlan {
+    std::vector<ResTile> tiles;  // none: no plan
+    size_t smem = 0;
+    int rows = 0;  // of the tallest tile
+};
+
+// The tiles of a handle's lattices if each block of a launch of at most
+// `blocks` can keep one: the flattest tiles that fit.  Flat tiles spread the
+// rows over all SMs, and a step is latency: 256^2 takes 2.73 us a step in 260
+// tiles of 4 rows, 2.95 in 145 of 8 and 4.3 in 60 of 21.
+inline ResPlan plan_resident(const std::vector<LatDev>& lats, int blocks, int es) {
+    ResPlan P;
+    const int most = res_rows(es);
+    int h = 0;  // the smallest height whose tiles fit
+    for (int rows = 2; rows <= most && !h; ++rows) {
+        int64_t n = 0;
+        int tallest = 0;
+        for (const LatDev& L : lats) {
+            const int nb = res_bands(L.ny, rows);
+            n += (int64_t)strip_count(L.nx) * nb;
+            tallest = std::max(tallest, (L.ny + nb - 1) / nb);
+            if (n > blocks) break;
+        }
+        if (n <= blocks && tallest <= most) {
+            h = rows;
+            P.smem = res_smem(tallest, kRowCols, es);
+            P.rows = tallest;
+        }
+    }
+    if (!h) return P;
+    for (size_t l = 0; l < lats.size(); ++l) {
+        const int nx = lats[l].nx, ny = lats[l].ny;
+        const int ns = strip_count(nx), nb = res_bands(ny, h), t0 = (int)P.tiles.size();
+        auto width = [&](int s) {
+            s = (s + ns) % ns;
+            return strip_edge(nx, ns, s + 1) - strip_edge(nx, ns, s);
+        };
+        auto groups = [&](int b) {
+            b = (b + nb) % nb;
+            return (band_edge(ny, nb, b + 1) - band_edge(ny, nb, b) + 2) / 3;
+        };
+        for (int s = 0; s < ns; ++s)
+            for (int b = 0; b < nb; ++b) {
+                ResTile t{};
+                t.lattice = (int)l;
+                t.x0 = strip_edge(nx, ns, s);
+                t.wd = width(s);
+                t.y0 = band_edge(ny, nb, b);
+                t.rows = band_edge(ny, nb, b + 1) - t.y0;
+                int k = 0;
+                for (int db = -1; db <= 1; ++db)
+                    for (int ds = -1; ds <= 1; ++ds)
+                        if (ds || db)
+                            t.nbr[k++] = t0 + (s + ds + ns) % ns * nb + (b + db + nb) % nb;
+                t.wd_w = width(s - 1);
+                t.wd_e = width(s + 1);
+                t.gr_n = groups(b - 1);
+                t.gr_s = groups(b + 1);
+                P.tiles.push_back(t);
+            }
+    }
+    return P;
+}
+
+}  // namespace pplbm

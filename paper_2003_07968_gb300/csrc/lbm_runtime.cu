@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <list>
 #include <map>
 #include <mutex>
 #include <new>
@@ -63,6 +64,28 @@ struct Pass {
 std::mutex g_tune_mu;
 std::map<TuneKey, TuneVal> g_tune_cache;
 
+// The resident launches in flight on a device.  Their blocks wait for one
+// another, so all blocks of every such launch that may run at the same time
+// must fit the GPU together: a launch goes ahead beside the others only while
+// their blocks and its own fit, and else waits (on the device) for the
+// longest-standing ones.  One entry a stream (a stream runs one launch at a
+// time): its last launch's end and the most blocks of its launches in flight.
+struct Flight {
+    cudaStream_t stream;
+    cudaEvent_t done;
+    int blocks;
+};
+struct Flights {
+    std::mutex mu;
+    std::list<Flight> list;  // the stream that launched last at the end
+};
+Flights& flights_of(int device) {
+    static std::mutex mu;
+    static std::map<int, Flights> all;
+    std::lock_guard<std::mutex> lk(mu);
+    return all[device];
+}
+
 }  // namespace
 
 struct lbm_handle {
@@ -112,6 +135,13 @@ struct lbm_handle {
     // wide); else that kernel uses row copies
     CUtensorMap tmap[2]{};  // loads, stores
     bool has_tmap = false;
+    // the lattices as resident tiles, when they fit (plan_resident): tiles,
+    // mailboxes and epochs in one allocation
+    int res_grid = 0;  // tiles (0: no plan)
+    size_t res_smem = 0, res_bytes = 0;
+    int res_slot = 0;
+    void* res = nullptr;
+    bool res_reset = true;  // mailboxes and epochs must be cleared first
     // profiling
     bool prof = false;
     ProfRec rec[2];
@@ -282,6 +312,103 @@ cudaError_t launch_pass(lbm_handle* h, int k, const StepArgs& a, int grid) {
                                 h->stream);
 }
 
+// Tiles, mailboxes and epochs of the handle's resident plan in h->res.
+ResTile* res_tiles(lbm_handle* h) { return static_cast<ResTile*>(h->res); }
+size_t res_mail_off(const lbm_handle* h) {
+    return (size_t)round_up((int64_t)(h->res_grid * sizeof(ResTile)), 256);
+}
+size_t res_epoch_off(const lbm_handle* h) {
+    return res_mail_off(h) + (size_t)h->res_grid * 2 * h->res_slot * sizeof(uint4);
+}
+
+// Plan the handle's lattices as resident tiles.  LBM_OK without a plan too.
+int make_resident(lbm_handle* h) {
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess || !coop)
+        return LBM_OK;
+    const ResPlan P = plan_resident(h->lat, std::min(2 * h->sm_count, kResBlocks), h->f16 ? 2 : 4);
+    if (P.tiles.empty()) return LBM_OK;
+    const int per_sm = resident_blocks_per_sm(h->f16, h->collision == LBM_COLL_MRT,
+                                              h->lat.size() == 1, P.smem);
+    if (per_sm < 2) return LBM_OK;  // the flights are counted at two blocks an SM
+    h->res_grid = (int)P.tiles.size();
+    h->res_smem = P.smem;
+    h->res_slot = res_packets(P.rows, kRowCols);
+    h->res_bytes = res_epoch_off(h) + h->res_grid * sizeof(uint32_t);
+    h->res = dev_alloc(h, h->res_bytes);
+    if (!h->res) return LBM_ERR_OOM;
+    CK(h, cudaMemcpyAsync(h->res, P.tiles.data(), P.tiles.size() * sizeof(ResTile),
+                          cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    return LBM_OK;
+}
+
+// nsteps steps in one launch (state from buffer `parity` to the other).
+// LBM_PENDING (nothing launched, no plan any more) where the device grants
+// this process fewer SMs than the plan needs.
+int launch_resident_steps(lbm_handle* h, int nsteps) {
+    if (h->res_reset) {
+        CK(h, cudaMemsetAsync(static_cast<char*>(h->res) + res_mail_off(h), 0,
+                              h->res_bytes - res_mail_off(h), h->stream));
+        h->res_reset = false;
+    }
+    ResArgs m{};
+    m.a = step_args(h, h->parity, 1);
+    m.tiles = res_tiles(h);
+    m.mail = reinterpret_cast<uint4*>(static_cast<char*>(h->res) + res_mail_off(h));
+    m.epoch = reinterpret_cast<uint32_t*>(static_cast<char*>(h->res) + res_epoch_off(h));
+    m.slot = h->res_slot;
+    m.nsteps = nsteps;
+    Flights& F = flights_of(h->device);
+    std::lock_guard<std::mutex> lk(F.mu);
+    auto mine = F.list.end();
+    for (auto it = F.list.begin(); it != F.list.end();) {
+        const cudaError_t q = cudaEventQuery(it->done);
+        if (q == cudaSuccess) {
+            cudaEventDestroy(it->done);
+            it = F.list.erase(it);
+            continue;
+        }
+        if (q != cudaErrorNotReady) return cuda_fail(h, q, "cudaEventQuery");
+        if (it->stream == h->stream) mine = it;
+        ++it;
+    }
+    // beside which of the other streams' launches it fits, the newest first
+    int room = 2 * h->sm_count - h->res_grid;
+    bool fits = true;
+    for (auto it = F.list.rbegin(); it != F.list.rend(); ++it) {
+        if (it->stream == h->stream) continue;
+        fits = fits && it->blocks <= room;
+        if (fits)
+            room -= it->blocks;
+        else
+            CK(h, cudaStreamWaitEvent(h->stream, it->done, 0));
+    }
+    if (mine == F.list.end()) {
+        Flight f{h->stream, nullptr, 0};
+        CK(h, cudaEventCreateWithFlags(&f.done, cudaEventDisableTiming));
+        mine = F.list.insert(F.list.end(), f);
+    } else {
+        F.list.splice(F.list.end(), F.list, mine);
+    }
+    const cudaError_t e =
+        launch_resident(h->f16, h->collision == LBM_COLL_MRT, m,
+                        h->lat.size() == 1 ? &h->lat[0] : nullptr, h->res_grid, h->res_smem, h->stream);
+    if (e == cudaSuccess) mine->blocks = std::max(mine->blocks, h->res_grid);
+    // (a record after a failed launch only marks the work queued before it)
+    const cudaError_t r = cudaEventRecord(mine->done, h->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {
+        cudaGetLastError();
+        h->res_grid = 0;
+        return r == cudaSuccess ? LBM_PENDING : cuda_fail(h, r, "cudaEventRecord");
+    }
+    if (e != cudaSuccess) return cuda_fail(h, e, "resident launch");
+    if (r != cudaSuccess) return cuda_fail(h, r, "cudaEventRecord");
+    h->launches += 1;
+    h->parity ^= 1;
+    return LBM_OK;
+}
+
 cudaEvent_t take_event(lbm_handle* h) {
     if (!h->ev_pool.empty()) {
         cudaEvent_t e = h->ev_pool.back();
@@ -427,6 +554,7 @@ void release(lbm_handle* h) {
         if (e) cudaEventDestroy(e);
     if (h->side) cudaStreamDestroy(h->side);
     for (auto& P : h->pass) dev_free(h, P.tiles, P.cap);
+    dev_free(h, h->res, h->res_bytes);
     dev_free(h, h->status, h->lat.size() * sizeof(uint32_t));
     dev_free(h, h->lat_dev, h->lat.size() * sizeof(LatDev));
     dev_free(h, h->psi, h->psi_bytes);
@@ -855,6 +983,13 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         if (cfg[q].grid > 0) h->pass[q].grid = std::min(cfg[q].grid, h->pass[q].ntiles);
         if (opts && opts->grid_ctas) h->pass[q].grid = std::min(opts->grid_ctas, h->pass[q].ntiles);
     }
+    // LBM_KERNEL_AUTO, float-float EOS: lattices that fit the SMs' shared memory
+    // are advanced many steps a launch (k_resident)
+    if (fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF && h->graph_steps > 0 &&
+        !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
+        const int rc = make_resident(h);
+        if (rc) return fail(rc);
+    }
     h->tune_variant = variant;
     h->rec[0].name = "psi_pass";
     h->rec[1].name = h->schedule == LBM_SCHED_FUSED ? "fused_step" : "collide_stream";
@@ -910,6 +1045,8 @@ static int lbm_init_body(lbm_handle* h, int32_t lattice, const double* rho, cons
                       h->stream));
     h->launches += 1;
     CK(h, cudaMemsetAsync(h->status + lattice, 0, sizeof(uint32_t), h->stream));
+    // a resident launch whose waits ran out leaves its tiles' epochs unequal
+    h->res_reset = true;
     if (h->numeric_lattice == lattice) {
         h->numeric_lattice = -1;
         h->fault_bits = 0;
@@ -927,6 +1064,21 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     int rc = check_status_async(h);
     if (rc) return rc;
     int64_t left = nsteps;
+    // resident lattices: from two steps on (one step is one tile-kernel launch;
+    // a resident one costs about 3 us beside its steps).  Not into a caller's
+    // stream capture: a replayed graph would not be counted among the flights.
+    if (h->res_grid && left >= 2 && !h->prof && !h->starve) {
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(h, cudaStreamIsCapturing(h->stream, &cap));
+        while (cap == cudaStreamCaptureStatusNone && left >= 2) {
+            // at most 2^14 steps a launch (a fraction of a second)
+            const int n = (int)std::min<int64_t>(left, left == (1 << 14) + 1 ? 1 << 13 : 1 << 14);
+            rc = launch_resident_steps(h, n);
+            if (rc == LBM_PENDING) break;
+            if (rc) return rc;
+            left -= n;
+        }
+    }
     if (!h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps) {
         if (!h->graph[h->parity]) {
             rc = capture_graph(h);

@@ -1,0 +1,104 @@
+"""The many-steps launch (k_resident) against one launch per step.
+
+A default handle whose lattices fit the SMs' shared memory advances many
+steps in one launch; graph_steps=-1 keeps it on the tile kernel, one launch
+per step.  Both run the same operations on the same values, so every output
+is equal bit for bit.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2003_07968_gb300 import build, capi
+
+    build.build()
+    capi.load()
+    return capi
+
+
+def _desc(P, nx, ny, storage, mrt, T=0.8, **kw):
+    if mrt:
+        kw.update(collision=P.LBM_COLL_MRT, tau=0.7, mrt_rates=[1.0] * 7 + [1.0 / 0.7] * 2)
+    return P.lbm_desc_default(nx, ny, T=T, storage=storage, **kw)
+
+
+def _field(nx, ny, k=0):
+    rng = np.random.default_rng(17 + k)
+    rho = synth.droplet(nx, ny, 0.3 * min(nx, ny) + 1, 0.8)
+    return rho + 1e-3 * rng.standard_normal(rho.shape)
+
+
+def _run(P, descs, fields, chunks, **kw):
+    h = P.lbm_create(descs, **kw)
+    for i, f in enumerate(fields):
+        P.lbm_init(h, i, f)
+    l0 = P.lbm_launch_count(h)
+    for n in chunks:
+        P.lbm_step(h, n)
+    launches = P.lbm_launch_count(h) - l0
+    out = [P.lbm_moments(h, i) for i in range(len(fields))]
+    P.lbm_destroy(h)
+    return out, launches
+
+
+def _same(a, b):
+    for x, y in zip(a, b):
+        for k in ("rho", "ux", "uy"):
+            assert np.array_equal(x[k], y[k]), k
+        assert x["mass"] == y["mass"]
+
+
+# edges of strips (60 columns), of rounds (8 rows) and of packets (3 values),
+# the narrowest lattices, the largest of the FP32 range
+SHAPES = [(2, 2), (3, 5), (5, 3), (60, 8), (61, 9), (119, 31), (120, 33), (121, 34), (64, 64),
+          (203, 77), (7, 150), (1500, 4), (181, 181), (777, 611)]
+
+
+@pytest.mark.parametrize("storage,mrt", [(1, 0), (0, 1), (2, 0), (2, 1)])
+def test_many_steps_equal_single_launches(P, storage, mrt):
+    for nx, ny in SHAPES:
+        d, f = _desc(P, nx, ny, storage, mrt, sigma=0.5), _field(nx, ny)
+        chunks = (2, 1, 3, 17)
+        a, la = _run(P, [d], [f], chunks)
+        b, lb = _run(P, [d], [f], chunks, graph_steps=-1)
+        assert (la, lb) == (4, 23), (nx, ny)
+        _same(a, b)
+
+
+def test_batches_of_resident_lattices(P):
+    sizes = [(64, 64), (2, 3), (130, 40), (61, 100), (33, 7)]
+    descs = [_desc(P, nx, ny, 1, 0, T=0.75 + 0.03 * k) for k, (nx, ny) in enumerate(sizes)]
+    descs[2] = _desc(P, 130, 40, 1, 0, T=0.9, eos_kind=P.LBM_EOS_KIND_VDW)
+    fields = [_field(nx, ny, k) for k, (nx, ny) in enumerate(sizes)]
+    fields[2] = synth.droplet(130, 40, 12.0, 0.9, densities=(0.42574, 1.65727))
+    a, la = _run(P, descs, fields, (40,))
+    b, lb = _run(P, descs, fields, (40,), graph_steps=-1)
+    assert (la, lb) == (1, 40)
+    _same(a, b)
+
+
+def test_handles_on_many_streams_at_once(P):
+    # blocks of a launch wait for one another, so launches that could run at
+    # the same time must fit the GPU together: handles that do not are queued
+    sizes = [(400, 400), (64, 64), (256, 256), (500, 300), (64, 64), (200, 200), (400, 410), (90, 90)]
+    hs = [P.lbm_create(_desc(P, nx, ny, 1, 0)) for nx, ny in sizes]
+    for k, (h, (nx, ny)) in enumerate(zip(hs, sizes)):
+        P.lbm_init(h, 0, _field(nx, ny, k))
+    for n in (50, 2, 101):
+        for h in hs:
+            P.lbm_step(h, n)
+    got = [P.lbm_moments(h, 0) for h in hs]
+    for h in hs:
+        P.lbm_destroy(h)
+    for k, (nx, ny) in enumerate(sizes):
+        want, _ = _run(P, [_desc(P, nx, ny, 1, 0)], [_field(nx, ny, k)], (153,), graph_steps=-1)
+        _same([got[k]], want)
