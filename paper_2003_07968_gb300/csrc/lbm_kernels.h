@@ -72,6 +72,9 @@ cudaError_t launch_fused_tma(int f16, int mrt, int eos, int tx, int ty, const St
                              const CUtensorMap* map, const LatDev* lat0, int grid,
                              cudaStream_t st);
 int occupancy_fused_tma(int f16, int mrt, int eos, int tx, int ty, bool with_map, bool single);
+// One step, a warp an item (a.tiles: row items, lbm_rows_plan.h; float-float
+// EOS); lat0 as in launch_fused_tma.
+cudaError_t launch_rows(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st);
 // Many steps in one cooperative launch over a resident plan's tiles
 // (float-float EOS; lbm_rows.cuh): lat0 as in launch_fused_tma.  All blocks
 // must be resident together: grid at most SMs x resident_blocks_per_sm.

@@ -7,6 +7,13 @@ namespace pplbm {
 cudaError_t resident_f32(int, const ResArgs*, const LatDev*, int, size_t, cudaStream_t, int*);
 cudaError_t resident_f16(int, const ResArgs*, const LatDev*, int, size_t, cudaStream_t, int*);
 
+cudaError_t rows_f32(int, const StepArgs&, const LatDev*, cudaStream_t);
+cudaError_t rows_f16(int, const StepArgs&, const LatDev*, cudaStream_t);
+
+cudaError_t launch_rows(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    return (f16 ? rows_f16 : rows_f32)(mrt, a, lat0, st);
+}
+
 cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
                             size_t smem, cudaStream_t st) {
     return (f16 ? resident_f16 : resident_f32)(mrt, &m, lat0, grid, smem, st, nullptr);

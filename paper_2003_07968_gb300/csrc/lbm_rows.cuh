@@ -161,6 +161,105 @@ __device__ __forceinline__ Strip strip_of(int x0, int xend, int pitch, int gx) {
     return s;
 }
 
+// ---------------------------------------------------------------- one step a launch
+// What a warp pulls for row y of its columns, from global memory (row: the
+// pair's place in row y of plane 0).
+template <class S>
+__device__ __forceinline__ void load_g(typename PairIO<S>::Raw g[9], const typename S::T* row,
+                                       int64_t plane, int pitch) {
+#pragma unroll
+    for (int i = 1; i < 9; ++i)
+        g[i] = PairIO<S>::ld(row + i * plane - (int64_t)plane_cy(i) * pitch);
+}
+
+// entry of a row-item list: (lattice, x0, y0, rows | width << 24)
+__device__ __forceinline__ int item_rows(int w) { return w & 0xffffff; }
+__device__ __forceinline__ int item_width(int w) { return w >> 24; }
+
+// k_rows: one step; every warp marches down the rows of an item of its own,
+// with no shared memory and no barrier.  Row y's values are loaded one row
+// ahead into registers; its pulled state and psi are computed, psi's row goes
+// to the neighbouring lanes by shuffles, and row y - 1, whose state waited in
+// registers, is collided and stored.  An item of h rows computes psi for
+// h + 2 and reads h + 4; a tile kernel's 32 x 16 tile computes it for 18 x 34
+// sites, fetches 20 x 40 and holds its warps at a barrier per tile.
+//
+// What bounds it: FP16 storage the FP32 pipe (75 % of its cycles; 61 % of
+// issue slots; paired instructions take two cycles), FP32 storage beyond L2
+// DRAM.  Measured per step, tile kernel (32 x 16) -> this one:
+//   FP16       4096^2 244 -> 190 us, 8192^2 937 -> 688 us (97.6 GLUPS);
+//              MRT 288 -> 230 and 1112 -> 846 us
+//   FP32 BGK   900^2 16.5 -> 14.9, 1200^2 33.4 -> 22.8, 433 x 2918 22.4 -> 22.3;
+//              2000^2 57 -> 64, 4096^2 222 -> 235 (the tile kernel's bulk
+//              copies keep DRAM busier), 8192^2 878 -> 835-868 us
+//   FP32 MRT   4096^2 255 -> 246, 8192^2 987 -> 896 us
+// Unrolling the row loop by 2 to save its register copies gained 4 % in FP16
+// BGK and spilled in the others (MRT 10 % slower); 5 blocks an SM spill too.
+template <class S, int EOSP, bool MRT, bool ONE>
+__global__ void __launch_bounds__(32 * kRowWarps, 4)
+    k_rows(StepArgs a, const __grid_constant__ LatDev lat0) {
+    using T = typename S::T;
+    using IO = PairIO<S>;
+    using Raw = typename IO::Raw;
+    __shared__ LatDev slat[ONE ? 1 : kRowWarps];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    (void)lane;
+    for (int t = blockIdx.x * kRowWarps + w; t < a.ntiles; t += gridDim.x * kRowWarps) {
+        const int4 tl = __ldg(&a.tiles[t]);
+        if (a.quota && a.step >= __ldg(&a.quota[tl.x])) continue;
+        if (!ONE) {
+            // the lattice's constants, in the warp's own copy
+            __syncwarp();
+            for (int k = lane; k < (int)(sizeof(LatDev) / 4); k += 32)
+                reinterpret_cast<int*>(&slat[w])[k] = __ldg(reinterpret_cast<const int*>(a.lats + tl.x) + k);
+            __syncwarp();
+        }
+        const LatDev& L = ONE ? lat0 : slat[w];
+        const SiteConsts C = site_consts(L);
+        const int nx = L.nx, ny = L.ny, pitch = L.pitch, gx = L.gx;
+        const int64_t plane = L.plane;
+        const int x0 = tl.y, y0 = tl.z, y1 = tl.z + item_rows(tl.w), xend = x0 + item_width(tl.w);
+        const Strip sp = strip_of(x0, xend, pitch, gx);
+        // row y0 - 1 of plane 0 (the first row whose psi is needed)
+        const T* p = reinterpret_cast<const T*>(a.pop) + L.off_f[a.parity] +
+                     (int64_t)(y0 - 1 + GY) * pitch + gx + sp.xl;
+        T* q = reinterpret_cast<T*>(a.pop) + L.off_f[a.parity ^ 1] +
+               (int64_t)(y0 - 2 + GY) * pitch + gx + sp.x;
+        Row3 Rm = row3<S>(IO::ld(p - pitch)), Rc = row3<S>(IO::ld(p));
+        Raw gn[9], rn;
+        load_g<S>(gn, p, plane, pitch);
+        rn = IO::ld(p + pitch);
+        Site<float2> sprev{};
+        Row3 P0{}, P1{};
+        for (int y = y0 - 1; y <= y1; ++y) {
+            Raw g[9];
+#pragma unroll
+            for (int i = 1; i < 9; ++i) g[i] = gn[i];
+            const Row3 Rp = row3<S>(rn);
+            p += pitch;
+            if (y < y1) {
+                load_g<S>(gn, p, plane, pitch);
+                rn = IO::ld(p + pitch);
+            }
+            const Site<float2> s = row_site<S>(g, Rm, Rc, Rp);
+            const Row3 P2 = row3(Eos<EOSP>::psi(L, site_rho(s, L.rho0), a.status, sp.live));
+            if (y > y0) {
+                const int ys = y - 1;
+                float2 v[9];
+                row_collide<S, MRT>(C, L.mrt_s, sprev, P0, P1, P2, v);
+                row_store<S>(q, plane, pitch, sp.x, ys, nx, ny, sp.in0, sp.in1,
+                             x0 < GW || xend > nx - GW || ys < GW || ys >= ny - GW, v);
+            }
+            q += pitch;
+            sprev = s;
+            P0 = P1;
+            P1 = P2;
+            Rm = Rc;
+            Rc = Rp;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- resident lattices
 // 16-byte packets between blocks: three values and the step's tag, written
 // and read as one 128-bit access.
@@ -462,7 +561,22 @@ cudaError_t resident_inst(const ResArgs* m, const LatDev* lat0, int grid, size_t
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(32 * kResWarps), p, smem, st);
 }
 
+template <class S, bool MRT>
+cudaError_t rows_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    const unsigned grid = (unsigned)((a.ntiles + kRowWarps - 1) / kRowWarps);
+    if (lat0)
+        k_rows<S, EOS_DF, MRT, true><<<grid, 32 * kRowWarps, 0, st>>>(a, *lat0);
+    else
+        k_rows<S, EOS_DF, MRT, false><<<grid, 32 * kRowWarps, 0, st>>>(a, LatDev{});
+    return cudaGetLastError();
+}
+
 }  // namespace
+
+template <class S>
+cudaError_t rows_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    return mrt ? rows_inst<S, true>(a, lat0, st) : rows_inst<S, false>(a, lat0, st);
+}
 
 // One storage type: the launch (occ null), or its blocks per SM into *occ
 // (lat0 not null: one lattice).

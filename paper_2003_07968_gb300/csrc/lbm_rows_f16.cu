@@ -8,4 +8,8 @@ cudaError_t resident_f16(int mrt, const ResArgs* m, const LatDev* lat0, int grid
     return resident_any<StoreF16>(mrt, m, lat0, grid, smem, st, occ);
 }
 
+cudaError_t rows_f16(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    return rows_any<StoreF16>(mrt, a, lat0, st);
+}
+
 }  // namespace pplbm

@@ -19,6 +19,50 @@ inline int strip_edge(int nx, int n, int k) {
 inline int strip_count(int nx) { return (nx + kRowCols - 1) / kRowCols; }
 inline int band_edge(int ny, int n, int k) { return (int)((int64_t)ny * k / n); }
 
+// ---- one step a launch (k_rows): row items, each the work of one warp
+constexpr int kRowWarps = 4;  // warps of a block, each on an item of its own
+// entry of an item list: (lattice, x0, y0, rows | width << 24)
+inline int pack_rows(int rows, int width) { return rows | (width << 24); }
+
+// Rows of an item: one wave of the `warps` the GPU holds where that makes
+// items of at most 16 rows (a second, partly filled wave costs more than the
+// three extra rows an item pulls and computes psi for), else about five
+// waves, of at most 64 rows.
+inline int row_item_height(const std::vector<LatDev>& lats, int64_t warps) {
+    int64_t units = 0;
+    for (const LatDev& L : lats) units += (int64_t)strip_count(L.nx) * L.ny;
+    for (int h = 2; h <= 16; ++h) {
+        int64_t n = 0;
+        for (const LatDev& L : lats) n += (int64_t)strip_count(L.nx) * ((L.ny + h - 1) / h);
+        if (n <= warps) return h;
+    }
+    return (int)std::min<int64_t>(64, std::max<int64_t>(8, units / (5 * warps)));
+}
+// Whether a step of these lattices runs on k_rows rather than on the tile
+// kernel (measured, see k_rows): FP16 storage always; FP32 where one wave of
+// warps covers the lattices (up to about 2.3 M sites), and again for one
+// lattice so large that both read DRAM evenly (MRT, whose arithmetic weighs
+// more, from half that on).
+inline bool rows_beat_tiles(const std::vector<LatDev>& lats, bool f16, bool mrt, int64_t warps) {
+    if (f16) return true;
+    int64_t items = 0;
+    for (const LatDev& L : lats) items += (int64_t)strip_count(L.nx) * ((L.ny + 15) / 16);
+    if (items <= warps) return true;
+    const int64_t sites = (int64_t)lats[0].nx * lats[0].ny;
+    return lats.size() == 1 && sites >= (int64_t)1 << (mrt ? 24 : 25);
+}
+// The items of one lattice, bands one after another, a band's strips side by side.
+inline void row_items(const LatDev& L, int lattice, int h, std::vector<int4>& out) {
+    const int ns = strip_count(L.nx), nb = (L.ny + h - 1) / h;
+    for (int b = 0; b < nb; ++b) {
+        const int y0 = band_edge(L.ny, nb, b), y1 = band_edge(L.ny, nb, b + 1);
+        for (int s = 0; s < ns; ++s) {
+            const int x0 = strip_edge(L.nx, ns, s), x1 = strip_edge(L.nx, ns, s + 1);
+            out.push_back(make_int4(lattice, x0, y0, pack_rows(y1 - y0, x1 - x0)));
+        }
+    }
+}
+
 // ---- resident lattices: one tile a block, kept in shared memory for many steps
 constexpr int kResWarps = 8;            // warps of a block, one row each at a time
 constexpr int kResSmem = 113 * 1024;    // shared memory of a block (two on an SM)

@@ -49,6 +49,7 @@ struct PassCfg {
 };
 struct TuneVal {
     PassCfg pass[2];
+    bool rows = false;  // the single pass: k_rows beat the best tile kernel
 };
 
 // One pass of the step (0: psi, 1: force + collision + stream): its kernel
@@ -135,6 +136,11 @@ struct lbm_handle {
     // wide); else that kernel uses row copies
     CUtensorMap tmap[2]{};  // loads, stores
     bool has_tmap = false;
+    // row items of the lattices for k_rows, and whether a step uses them
+    int4* items = nullptr;
+    int n_items = 0;
+    size_t items_bytes = 0;
+    bool rows = false;
     // the lattices as resident tiles, when they fit (plan_resident): tiles,
     // mailboxes and epochs in one allocation
     int res_grid = 0;  // tiles (0: no plan)
@@ -343,6 +349,28 @@ int make_resident(lbm_handle* h) {
     return LBM_OK;
 }
 
+// Row items of the handle's lattices.
+int make_items(lbm_handle* h) {
+    const int height = row_item_height(h->lat, (int64_t)h->sm_count * 4 * kRowWarps);
+    std::vector<int4> t;
+    for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, height, t);
+    h->items_bytes = t.size() * sizeof(int4);
+    h->items = (int4*)dev_alloc(h, h->items_bytes);
+    if (!h->items) return LBM_ERR_OOM;
+    CK(h, cudaMemcpyAsync(h->items, t.data(), h->items_bytes, cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    h->n_items = (int)t.size();
+    return LBM_OK;
+}
+
+cudaError_t launch_row_step(lbm_handle* h, int parity) {
+    StepArgs a = step_args(h, parity, 1);
+    a.tiles = h->items;
+    a.ntiles = h->n_items;
+    return launch_rows(h->f16, h->collision == LBM_COLL_MRT, a,
+                       h->lat.size() == 1 ? &h->lat[0] : nullptr, h->stream);
+}
+
 // nsteps steps in one launch (state from buffer `parity` to the other).
 // LBM_PENDING (nothing launched, no plan any more) where the device grants
 // this process fewer SMs than the plan needs.
@@ -439,7 +467,10 @@ int launch_step(lbm_handle* h, int p) {
     a1.starve = h->starve;  // an armed failure-detection test goes into this launch only
     if (h->starve) a1.wait_cycles = kTestWaitBudgetCycles;
     h->starve = 0;
-    CK(h, launch_pass(h, 1, a1, h->pass[1].grid));
+    if (h->rows && !a1.starve)
+        CK(h, launch_row_step(h, p));
+    else
+        CK(h, launch_pass(h, 1, a1, h->pass[1].grid));
     if (h->prof) {
         CK(h, cudaEventRecord(e2, h->stream));
         // the psi pair owns e0, the step pair owns e1 and e2
@@ -555,6 +586,7 @@ void release(lbm_handle* h) {
     if (h->side) cudaStreamDestroy(h->side);
     for (auto& P : h->pass) dev_free(h, P.tiles, P.cap);
     dev_free(h, h->res, h->res_bytes);
+    dev_free(h, h->items, h->items_bytes);
     dev_free(h, h->status, h->lat.size() * sizeof(uint32_t));
     dev_free(h, h->lat_dev, h->lat.size() * sizeof(LatDev));
     dev_free(h, h->psi, h->psi_bytes);
@@ -957,13 +989,17 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         if (fused_tma_make_map(h->f16, 32, 16, h->lat.data(), n, h->pop, probe))
             cfg[1] = PassCfg{LBM_KERNEL_TMA, 32, 16, 0, 2};
     }
+    bool tuned = false, tuned_rows = false;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         TuneKey k{h->device, h->storage, h->eos, variant * 4 + h->schedule,
                   (int64_t)std::log2((double)h->sites), (int64_t)std::log2((double)n)};
         auto it = g_tune_cache.find(k);
-        if (it != g_tune_cache.end() && !(opts && (opts->tile_x || opts->tile_y)))
+        if (it != g_tune_cache.end() && !(opts && (opts->tile_x || opts->tile_y))) {
             for (int q = 0; q < 2; ++q) cfg[q] = it->second.pass[q];
+            tuned = true;
+            tuned_rows = it->second.rows;
+        }
     }
     if (cfg[1].variant == LBM_KERNEL_TMA &&
         !shape_ok(LBM_KERNEL_TMA, cfg[1].tx, cfg[1].ty, 1, fused))
@@ -989,6 +1025,15 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
         const int rc = make_resident(h);
         if (rc) return fail(rc);
+    }
+    // ... and single steps may run on k_rows
+    if (fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
+        !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
+        const int rc = make_items(h);
+        if (rc) return fail(rc);
+        h->rows = tuned ? tuned_rows
+                        : rows_beat_tiles(h->lat, h->f16, h->collision == LBM_COLL_MRT,
+                                          (int64_t)h->sm_count * 4 * kRowWarps);
     }
     h->tune_variant = variant;
     h->rec[0].name = "psi_pass";
@@ -1348,6 +1393,18 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
         rc = build_tiles(h, k, bc.tx, bc.ty);
         h->pass[k].grid = bc.grid;
         best_cfg.pass[k] = bc;
+        if (k == 1 && h->items && rc == LBM_OK) {
+            // the row kernel against the best tile kernel
+            cudaError_t e = launch_row_step(h, h->parity);  // warm-up
+            cudaEventRecord(ea, h->stream);
+            for (int r = 0; r < repeats && e == cudaSuccess; ++r) e = launch_row_step(h, h->parity);
+            cudaEventRecord(eb, h->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(eb);
+            if (e != cudaSuccess) { rc = cuda_fail(h, e, "autotune rows"); break; }
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, ea, eb);
+            best_cfg.rows = h->rows = ms < best;
+        }
     }
     cudaEventDestroy(ea);
     cudaEventDestroy(eb);

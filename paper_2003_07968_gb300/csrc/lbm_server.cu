@@ -186,6 +186,7 @@ struct lbm_server {
     float* psi_arena = nullptr;
     int64_t pitch = 0, plane = 0, row_cap = 0;  // of the row space (elements, rows)
     size_t pop_bytes = 0, psi_region = 0;
+    bool rows = false;     // single pass on the row kernel (FP16 storage; tile lists are row items)
     bool tma = false;      // single pass on the TMA kernel (one tensor map for the arena)
     CUtensorMap tmap[2]{};  // loads, stores
     size_t up_cap = 0;            // doubles of the device staging buffer
@@ -295,6 +296,7 @@ cudaError_t launch(lbm_server* S, int k, const StepArgs& a, int grid, cudaStream
     const PassState& P = S->pass[k];
     const dim3 block(P.tx, P.ty / P.spt);
     if (k == 0) return launch_psi(S->f16, S->o.eos_precision, P.spt, a, dim3(grid), block, st);
+    if (S->rows) return launch_rows(S->f16, 0, a, nullptr, st);
     if (S->tma)
         return launch_fused_tma(S->f16, 0, S->o.eos_precision, P.tx, P.ty, a, S->tmap, nullptr,
                                 grid, st);
@@ -346,9 +348,18 @@ cudaError_t rebuild(lbm_server* S, TableSet& T, std::vector<Request*>& res,
     if (e != cudaSuccess) return e;
     for (int k = 0; k < 2; ++k) {
         const PassState& P = S->pass[k];
+        const bool items = k == 1 && S->rows;
         size_t nt = 0;
+        std::vector<int4> rt;
+        if (items) {
+            std::vector<LatDev> lats;
+            for (Request* R : res) lats.push_back(R->L);
+            const int height = row_item_height(lats, (int64_t)S->sm_count * 4 * kRowWarps);
+            for (size_t l = 0; l < res.size(); ++l) row_items(lats[l], (int)l, height, rt);
+            nt = rt.size();
+        }
         for (Request* R : res)
-            nt += (size_t)((R->L.nx + P.tx - 1) / P.tx) * ((R->L.ny + P.ty - 1) / P.ty);
+            if (!items) nt += (size_t)((R->L.nx + P.tx - 1) / P.tx) * ((R->L.ny + P.ty - 1) / P.ty);
         const size_t bytes = nt * sizeof(int4);
         if (bytes > T.cap[k]) {
             if (T.tiles[k]) {
@@ -374,7 +385,8 @@ cudaError_t rebuild(lbm_server* S, TableSet& T, std::vector<Request*>& res,
         size_t m = 0;
         T.begin[k].assign(res.size(), 0);
         T.count[k].assign(res.size(), 0);
-        for (size_t l = 0; l < res.size(); ++l) {
+        if (items) std::copy(rt.begin(), rt.end(), t);
+        for (size_t l = 0; l < res.size() && !items; ++l) {
             T.begin[k][l] = (int)m;
             for (int y0 = 0; y0 < res[l]->L.ny; y0 += P.ty)
                 for (int x0 = 0; x0 < res[l]->L.nx; x0 += P.tx) t[m++] = make_int4((int)l, x0, y0, 0);
@@ -1008,6 +1020,10 @@ static int lbm_server_create_body(const lbm_server_opts* opts, lbm_server** out)
         S->pass[1].ty = kPassDefaults[1].ty;
         S->pass[1].spt = kPassDefaults[1].spt;
     }
+    // FP16 storage: the row kernel (see rows_beat_tiles; the resident lattices
+    // change from chunk to chunk, FP32 ones stay on the tile kernel)
+    S->rows = S->tma && S->f16 && o.kernel_variant == LBM_KERNEL_AUTO &&
+              o.eos_precision == LBM_EOS_DF && !(o.tile_x || o.tile_y);
     S->st.arena_bytes = (int64_t)o.arena_bytes;
     try {
         S->worker = std::thread(worker_main, S);

@@ -102,3 +102,54 @@ def test_handles_on_many_streams_at_once(P):
     for k, (nx, ny) in enumerate(sizes):
         want, _ = _run(P, [_desc(P, nx, ny, 1, 0)], [_field(nx, ny, k)], (153,), graph_steps=-1)
         _same([got[k]], want)
+
+
+# ------------------------------------------------------- one step a launch on rows
+# lattices beyond the resident range: edges of strips and items, ragged sizes,
+# the narrowest and the flattest, one wave of items and several
+ROW_SHAPES = [(901, 1403), (1200, 1100), (3, 40011), (61, 21001), (16001, 85), (2500, 1931)]
+
+
+@pytest.mark.parametrize("storage,mrt", [(1, 0), (1, 1), (2, 0), (2, 1)])
+def test_row_kernel_equals_tile_kernel(P, storage, mrt):
+    for nx, ny in ROW_SHAPES:
+        d, f = _desc(P, nx, ny, storage, mrt, sigma=0.5), _field(nx, ny)
+        a, la = _run(P, [d], [f], (5,))
+        b, lb = _run(P, [d], [f], (5,), kernel_variant=P.LBM_KERNEL_TMA)
+        assert la == lb == 5, (nx, ny)  # one launch a step: not resident
+        _same(a, b)
+
+
+@pytest.mark.parametrize("storage", [1, 2])
+def test_row_kernel_batches(P, storage):
+    sizes = [(700, 651), (3, 5), (61, 300), (800, 701), (33, 7), (640, 640)]
+    descs = [_desc(P, nx, ny, storage, 0, T=0.7 + 0.04 * k) for k, (nx, ny) in enumerate(sizes)]
+    fields = [_field(nx, ny, k) for k, (nx, ny) in enumerate(sizes)]
+    a, la = _run(P, descs, fields, (5,))
+    b, lb = _run(P, descs, fields, (5,), kernel_variant=P.LBM_KERNEL_TMA)
+    assert la == lb == 5
+    _same(a, b)
+
+
+def test_served_fp16_results_equal_a_plain_handle(P):
+    # the server's FP16 requests run on row items, with step quotas
+    import time
+
+    srv = P.lbm_server_create(P.lbm_server_opts_default(
+        arena_bytes=1 << 30, max_request_sites=512 * 512, max_width=512, chunk_steps=7,
+        storage=P.LBM_STORE_F16_DEV))
+    reqs = [(100, 37, 20), (512, 300, 31), (61, 130, 5), (2, 3, 9), (400, 512, 13)]
+    todo = {}
+    for k, (nx, ny, n) in enumerate(reqs):
+        d, f = _desc(P, nx, ny, P.LBM_STORE_F16_DEV, 0), _field(nx, ny, k)
+        todo[P.lbm_submit(srv, d, f, n)] = (d, f, n)
+    while todo:
+        for t in list(todo):
+            got = P.lbm_poll(srv, t)
+            if got is not None:
+                d, f, n = todo.pop(t)
+                want, _ = _run(P, [d], [f], (n,), kernel_variant=P.LBM_KERNEL_TMA)
+                for key in ("rho", "ux", "uy"):
+                    assert np.array_equal(got[key], want[0][key]), (key, d.nx, d.ny)
+        time.sleep(0.001)
+    P.lbm_server_destroy(srv)
