@@ -421,11 +421,18 @@ __device__ __forceinline__ void signed_sum(const float v[N], const int w[N], flo
     }
 }
 
-// Rows y0 .. y1 - 1; the output pointers point at row y0 of their fields.
+// Rows y0 .. y1 - 1; the output pointers point at row y0 of their fields, in
+// device memory or in the caller's page-locked arrays.  faults.n > 0: the
+// first block also copies that many fault words to the host (page-locked),
+// which saves lbm_moments a copy of its own.
 template <class S>
 __global__ void k_moments(LatDev L, const void* pop, int parity, const float* psi_arena,
-                          double* rho_out, double* ux_out, double* uy_out, int y0, int y1) {
+                          double* rho_out, double* ux_out, double* uy_out, int y0, int y1,
+                          FaultCopy faults) {
     using T = typename S::T;
+    if (faults.n && blockIdx.x == 0 && blockIdx.y == 0)
+        for (int i = threadIdx.y * blockDim.x + threadIdx.x; i < faults.n; i += blockDim.x * blockDim.y)
+            faults.to[i] = faults.from[i];
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = y0 + (int)(blockIdx.y * blockDim.y + threadIdx.y);
     const int nx = L.nx;
@@ -739,7 +746,7 @@ cudaError_t launch_init(int storage_f16, const LatDev& L, void* pop, int parity,
 
 cudaError_t launch_moments(int storage_f16, const LatDev& L, const void* pop, int parity,
                            const float* psi, double* rho, double* ux, double* uy, int y0, int y1,
-                           cudaStream_t st) {
+                           cudaStream_t st, FaultCopy faults) {
     if (y1 <= y0) return cudaSuccess;
     // rows y0 .. y1 - 1: the outputs' rows start at row y0 of the [ny][nx] fields
     dim3 b(32, 8), g((L.nx + 31) / 32, (y1 - y0 + 7) / 8);
@@ -748,9 +755,9 @@ cudaError_t launch_moments(int storage_f16, const LatDev& L, const void* pop, in
     double* u = ux ? ux + off : nullptr;
     double* v = uy ? uy + off : nullptr;
     if (storage_f16)
-        k_moments<StoreF16><<<g, b, 0, st>>>(L, pop, parity, psi, r, u, v, y0, y1);
+        k_moments<StoreF16><<<g, b, 0, st>>>(L, pop, parity, psi, r, u, v, y0, y1, faults);
     else
-        k_moments<StoreF32><<<g, b, 0, st>>>(L, pop, parity, psi, r, u, v, y0, y1);
+        k_moments<StoreF32><<<g, b, 0, st>>>(L, pop, parity, psi, r, u, v, y0, y1, faults);
     return cudaGetLastError();
 }
 

@@ -18,10 +18,16 @@ cudaError_t launch_collide(int storage_f16, int mrt, int spt, const StepArgs& a,
 cudaError_t launch_init(int storage_f16, const LatDev& L, void* pop, int parity,
                         const double* rho, const float* rho32, const double* ux, const double* uy,
                         cudaStream_t st);
+// Fault words to copy to page-locked host memory along with a field (n = 0: none).
+struct FaultCopy {
+    const uint32_t* from = nullptr;
+    uint32_t* to = nullptr;
+    int n = 0;
+};
 // rho, u of rows y0 .. y1 - 1 into [ny][nx] fields (any may be NULL).
 cudaError_t launch_moments(int storage_f16, const LatDev& L, const void* pop, int parity,
                            const float* psi, double* rho, double* ux, double* uy, int y0, int y1,
-                           cudaStream_t st);
+                           cudaStream_t st, FaultCopy faults = FaultCopy{});
 // The smallest of n device values into *out, or NaN if any is not finite
 // (partials: at least n_partials doubles of scratch); the values rounded to
 // FP32 into v32.

@@ -27,6 +27,7 @@ using namespace pplbm;
 namespace {
 
 constexpr int kMassPartials = 1024;
+constexpr size_t kDirectSites = (size_t)1 << 20;  // see lbm_moments
 
 struct ProfRec {
     std::string name;
@@ -124,6 +125,7 @@ struct lbm_handle {
     int numeric_lattice = -1;  // first lattice with a device fault bit
     uint32_t fault_bits = 0;   // OR of the device fault bits seen
     int sm_count = 0;
+    int host_access = 0;  // the device reaches all host memory (pageableMemoryAccess)
     int parity = 0;
     int64_t sites = 0;
     int64_t launches = 0;
@@ -343,9 +345,9 @@ int make_resident(lbm_handle* h) {
     h->res_bytes = res_epoch_off(h) + h->res_grid * sizeof(uint32_t);
     h->res = dev_alloc(h, h->res_bytes);
     if (!h->res) return LBM_ERR_OOM;
+    // (a copy from pageable memory has read it when the call returns)
     CK(h, cudaMemcpyAsync(h->res, P.tiles.data(), P.tiles.size() * sizeof(ResTile),
                           cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     return LBM_OK;
 }
 
@@ -358,7 +360,6 @@ int make_items(lbm_handle* h) {
     h->items = (int4*)dev_alloc(h, h->items_bytes);
     if (!h->items) return LBM_ERR_OOM;
     CK(h, cudaMemcpyAsync(h->items, t.data(), h->items_bytes, cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     h->n_items = (int)t.size();
     return LBM_OK;
 }
@@ -537,13 +538,32 @@ int check_status_async(lbm_handle* h) {
     return fault_code(h);
 }
 
-int sync_status(lbm_handle* h) {
+// Wait for the stream; `copied`: the fault words are on their way to
+// status_host already.
+int sync_status(lbm_handle* h, bool copied = false) {
+    if (!copied)
+        CK(h, cudaMemcpyAsync(h->status_host, h->status, h->lat.size() * sizeof(uint32_t),
+                              cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    CK(h, cudaMemcpy(h->status_host, h->status, h->lat.size() * sizeof(uint32_t),
-                     cudaMemcpyDeviceToHost));
     h->status_pending = false;
     absorb_status(h);
     return fault_code(h);
+}
+
+// The device's address of n host doubles that kernels may write themselves:
+// page-locked (both ends), on a device that reaches host memory coherently.
+// Null where a copy has to bring the field.
+double* host_direct(const lbm_handle* h, double* p, size_t n) {
+    if (!h->host_access || !p) return nullptr;
+    cudaPointerAttributes a{}, b{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
+        cudaPointerGetAttributes(&b, p + n - 1) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (a.type != cudaMemoryTypeHost || b.type != cudaMemoryTypeHost) return nullptr;
+    double* const d = static_cast<double*>(a.devicePointer);
+    return d && static_cast<double*>(b.devicePointer) == d + (n - 1) ? d : nullptr;
 }
 
 // Bytes of the staging buffer for fields of `elems` sites: three FP64 fields
@@ -936,6 +956,9 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
     if (cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device) !=
         cudaSuccess)
         return fail(LBM_ERR_CUDA);
+    if (cudaDeviceGetAttribute(&h->host_access, cudaDevAttrPageableMemoryAccess, h->device) !=
+        cudaSuccess)
+        return fail(LBM_ERR_CUDA);
     if (opts && opts->stream) {
         h->stream = (cudaStream_t)opts->stream;
     } else {
@@ -1026,8 +1049,8 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         const int rc = make_resident(h);
         if (rc) return fail(rc);
     }
-    // ... and single steps may run on k_rows
-    if (fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
+    // ... and larger ones may run on k_rows
+    if (!h->res_grid && fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
         !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
         const int rc = make_items(h);
         if (rc) return fail(rc);
@@ -1177,32 +1200,55 @@ static int lbm_moments_body(lbm_handle* h, int32_t lattice, double* rho, double*
     if (!h || lattice < 0 || lattice >= (int)h->lat.size()) return LBM_ERR_ARG;
     const LatDev& L = h->lat[lattice];
     const size_t n = (size_t)L.nx * L.ny;
-    if (rho || ux || uy) {
+    const bool vel = ux || uy;
+    // fields small enough that the copies' latency is most of the call: the
+    // kernel writes the caller's page-locked arrays (and the fault words)
+    // itself.  A density read back at 64^2 / 256^2 / 512^2 / 1024^2 took 28 / 32 /
+    // 49 / 82 us through a staging buffer, two copies and the events between
+    // two streams, and takes 15 / 17 / 26 / 58 us so.
+    double *hr = nullptr, *hx = nullptr, *hy = nullptr;
+    bool direct = (rho || vel) && n <= kDirectSites;
+    if (direct) {
+        hr = host_direct(h, rho, n);
+        hx = host_direct(h, ux, n);
+        hy = host_direct(h, uy, n);
+        direct = (!rho || hr) && (!ux || hx) && (!uy || hy);
+    }
+    if ((rho || vel) && !direct) {
         int rc = ensure_staging(h, n);
         if (rc) return rc;
-        // velocities: psi of the current state for this lattice's tiles (the
-        // force-shifted u needs the force); density alone needs neither
-        if (ux || uy) {
-            StepArgs a = step_args(h, h->parity, 0);
-            a.tiles = h->pass[0].tiles + h->pass[0].begin[lattice];
-            a.ntiles = h->pass[0].count[lattice];
-            CK(h, launch_pass(h, 0, a, std::min(h->pass[0].grid, a.ntiles)));
-            h->launches += 1;
-        }
     }
-    // The fields are computed in row chunks on the handle's stream; the side
+    // velocities: psi of the current state for this lattice's tiles (the
+    // force-shifted u needs the force); density alone needs neither
+    if (vel) {
+        StepArgs a = step_args(h, h->parity, 0);
+        a.tiles = h->pass[0].tiles + h->pass[0].begin[lattice];
+        a.ntiles = h->pass[0].count[lattice];
+        CK(h, launch_pass(h, 0, a, std::min(h->pass[0].grid, a.ntiles)));
+        h->launches += 1;
+    }
+    if (direct) {
+        FaultCopy faults;
+        faults.from = h->status;
+        faults.to = h->status_host;
+        faults.n = (int)h->lat.size();
+        CK(h, launch_moments(h->f16, L, h->pop, h->parity, h->psi, hr, hx, hy, 0, L.ny, h->stream,
+                             faults));
+        h->launches += 1;
+    }
+    // Larger fields are computed in row chunks on the handle's stream; the side
     // stream copies each finished chunk to the caller while the next chunk
     // and the mass reduction run.  The handle's stream then waits for the
     // copies, so nothing later reuses the staging buffer before they are done.
-    const int nchunk = (rho || ux || uy) ? (n >= ((size_t)1 << 22) ? 4 : 1) : 0;
+    const int nchunk = (rho || vel) && !direct ? (n >= ((size_t)1 << 22) ? 4 : 1) : 0;
     for (int c = 0; c < nchunk; ++c) {
         const int y0 = (int)((int64_t)L.ny * c / nchunk), y1 = (int)((int64_t)L.ny * (c + 1) / nchunk);
         const size_t off = (size_t)y0 * L.nx, cnt = (size_t)(y1 - y0) * L.nx;
         double* dr = h->staging;
         double* dx = h->staging + h->staging_elems;
         double* dy = h->staging + 2 * h->staging_elems;
-        CK(h, launch_moments(h->f16, L, h->pop, h->parity, h->psi, dr, (ux || uy) ? dx : nullptr,
-                             (ux || uy) ? dy : nullptr, y0, y1, h->stream));
+        CK(h, launch_moments(h->f16, L, h->pop, h->parity, h->psi, dr, vel ? dx : nullptr,
+                             vel ? dy : nullptr, y0, y1, h->stream));
         h->launches += 1;
         CK(h, cudaEventRecord(h->chunk_ev[c], h->stream));
         CK(h, cudaStreamWaitEvent(h->side, h->chunk_ev[c], 0));
@@ -1212,17 +1258,22 @@ static int lbm_moments_body(lbm_handle* h, int32_t lattice, double* rho, double*
         if (uy) CK(h, cudaMemcpyAsync(uy + off, dy + off, b, cudaMemcpyDeviceToHost, h->side));
     }
     if (mass) {
+        // (the result goes through the handle's page-locked word: a copy to
+        // pageable memory would wait for the stream by itself)
         CK(h, launch_mass(h->f16, L, h->pop, h->parity, h->partials, kMassPartials,
-                          h->partials + kMassPartials, h->stream));
+                          h->host_access ? h->scan_host : h->partials + kMassPartials, h->stream));
         h->launches += 2;
-        CK(h, cudaMemcpyAsync(mass, h->partials + kMassPartials, sizeof(double),
-                              cudaMemcpyDeviceToHost, h->stream));
+        if (!h->host_access)
+            CK(h, cudaMemcpyAsync(h->scan_host, h->partials + kMassPartials, sizeof(double),
+                                  cudaMemcpyDeviceToHost, h->stream));
     }
     if (nchunk) {
         CK(h, cudaEventRecord(h->chunk_ev[4], h->side));
         CK(h, cudaStreamWaitEvent(h->stream, h->chunk_ev[4], 0));
     }
-    return sync_status(h);
+    const int rc = sync_status(h, direct);
+    if (mass) *mass = *h->scan_host;
+    return rc;
 }
 
 int lbm_moments(lbm_handle* h, int32_t lattice, double* rho, double* ux, double* uy,

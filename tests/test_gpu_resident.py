@@ -153,3 +153,28 @@ def test_served_fp16_results_equal_a_plain_handle(P):
                     assert np.array_equal(got[key], want[0][key]), (key, d.nx, d.ny)
         time.sleep(0.001)
     P.lbm_server_destroy(srv)
+
+
+# ------------------------------------------------------------ fields read back
+def test_fields_read_back_into_any_host_array(P):
+    # page-locked arrays are written by the kernel itself up to 2^20 sites,
+    # others through copies: the same values, whichever each field lies in
+    import torch
+
+    for nx, ny in ((5, 3), (77, 41), (1024, 1024), (1025, 1024)):
+        h = P.lbm_create(_desc(P, nx, ny, 1, 0))
+        P.lbm_init(h, 0, _field(nx, ny))
+        P.lbm_step(h, 4)
+        pin = lambda: torch.full((ny, nx), -1.0, dtype=torch.float64, pin_memory=True).numpy()
+        page = lambda: np.full((ny, nx), -1.0)
+        want = P.lbm_moments(h, 0, out={k: page() for k in ("rho", "ux", "uy")})
+        # one field alone, an array inside a larger page-locked one, a mixture
+        big = torch.full((2 * ny * nx + 3,), -1.0, dtype=torch.float64, pin_memory=True).numpy()
+        rho = big[3:3 + nx * ny].reshape(ny, nx)
+        P.lbm_moments(h, 0, u=False, mass=False, out={"rho": rho})
+        assert np.array_equal(rho, want["rho"])
+        assert np.all(big[:3] == -1.0) and np.all(big[3 + nx * ny:] == -1.0)
+        for mix in ((pin(), pin(), pin()), (pin(), page(), pin())):
+            got = P.lbm_moments(h, 0, out=dict(zip(("rho", "ux", "uy"), mix)))
+            _same([got], [want])
+        P.lbm_destroy(h)
