@@ -129,6 +129,7 @@ struct StepArgs {
     // step >= quota[lattice] are skipped; nullptr for handles
     const int* quota;
     int step;
+    int last_only = 0;  // k_rows: only lattices whose quota ends with this step
     // failure-detection test: tile + 1 whose staging copy the single pass
     // skips, so that the consumers' bounded wait for it runs out (0: none)
     int starve = 0;

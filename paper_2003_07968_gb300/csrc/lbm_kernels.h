@@ -81,6 +81,9 @@ int occupancy_fused_tma(int f16, int mrt, int eos, int tx, int ty, bool with_map
 // One step, a warp an item (a.tiles: row items, lbm_rows_plan.h; float-float
 // EOS); lat0 as in launch_fused_tma.
 cudaError_t launch_rows(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st);
+// Two steps, a pair of warps an item (a.tiles: row items of kPairCols; float-
+// float EOS; lattices of less than 4 GB a plane).
+cudaError_t launch_pairs(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st);
 // Many steps in one cooperative launch over a resident plan's tiles
 // (float-float EOS; lbm_rows.cuh): lat0 as in launch_fused_tma.  All blocks
 // must be resident together: grid at most SMs x resident_blocks_per_sm.

@@ -14,6 +14,13 @@ cudaError_t launch_rows(int f16, int mrt, const StepArgs& a, const LatDev* lat0,
     return (f16 ? rows_f16 : rows_f32)(mrt, a, lat0, st);
 }
 
+cudaError_t pairs_f32(int, const StepArgs&, const LatDev*, cudaStream_t);
+cudaError_t pairs_f16(int, const StepArgs&, const LatDev*, cudaStream_t);
+
+cudaError_t launch_pairs(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    return (f16 ? pairs_f16 : pairs_f32)(mrt, a, lat0, st);
+}
+
 cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
                             size_t smem, cudaStream_t st) {
     return (f16 ? resident_f16 : resident_f32)(mrt, &m, lat0, grid, smem, st, nullptr);

@@ -9,6 +9,7 @@
 // The arithmetic is that of lbm_device.cuh, operation for operation, so every
 // result is bitwise that of the tile kernels.
 #pragma once
+#include "lbm_async.cuh"
 #include "lbm_kernels.h"
 #include "lbm_rows_plan.h"
 
@@ -189,10 +190,8 @@ __device__ __forceinline__ int item_width(int w) { return w >> 24; }
 // DRAM.  Measured per step, tile kernel (32 x 16) -> this one:
 //   FP16       4096^2 244 -> 190 us, 8192^2 937 -> 688 us (97.6 GLUPS);
 //              MRT 288 -> 230 and 1112 -> 846 us
-//   FP32 BGK   900^2 16.5 -> 14.9, 1200^2 33.4 -> 22.8, 433 x 2918 22.4 -> 22.3;
-//              2000^2 57 -> 64, 4096^2 222 -> 235 (the tile kernel's bulk
-//              copies keep DRAM busier), 8192^2 878 -> 835-868 us
-//   FP32 MRT   4096^2 255 -> 246, 8192^2 987 -> 896 us
+//   FP32 BGK   900^2 16.5 -> 14.9, 1200^2 33.4 -> 22.8; 4096^2 222 -> 235
+//              (there it takes the odd step beside k_rows2 only)
 // Unrolling the row loop by 2 to save its register copies gained 4 % in FP16
 // BGK and spilled in the others (MRT 10 % slower); 5 blocks an SM spill too.
 template <class S, int EOSP, bool MRT, bool ONE>
@@ -206,7 +205,10 @@ __global__ void __launch_bounds__(32 * kRowWarps, 4)
     (void)lane;
     for (int t = blockIdx.x * kRowWarps + w; t < a.ntiles; t += gridDim.x * kRowWarps) {
         const int4 tl = __ldg(&a.tiles[t]);
-        if (a.quota && a.step >= __ldg(&a.quota[tl.x])) continue;
+        if (a.quota) {
+            const int left = __ldg(&a.quota[tl.x]) - a.step;
+            if (left <= 0 || (a.last_only && left > 1)) continue;
+        }
         if (!ONE) {
             // the lattice's constants, in the warp's own copy
             __syncwarp();
@@ -248,6 +250,211 @@ __global__ void __launch_bounds__(32 * kRowWarps, 4)
                 float2 v[9];
                 row_collide<S, MRT>(C, L.mrt_s, sprev, P0, P1, P2, v);
                 row_store<S>(q, plane, pitch, sp.x, ys, nx, ny, sp.in0, sp.in1,
+                             x0 < GW || xend > nx - GW || ys < GW || ys >= ny - GW, v);
+            }
+            q += pitch;
+            sprev = s;
+            P0 = P1;
+            P1 = P2;
+            Rm = Rc;
+            Rc = Rp;
+        }
+    }
+}
+
+// ---------------------------------------------------------------- two steps a launch
+// A pair's raw value from two columns of a row.
+__device__ __forceinline__ float2 raw_of(float a, float b) { return make_float2(a, b); }
+__device__ __forceinline__ uint32_t raw_of(__half a, __half b) {
+    return (uint32_t)__half_as_ushort(a) | (uint32_t)__half_as_ushort(b) << 16;
+}
+__device__ __forceinline__ float ld_one(const float* p) {
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half ld_one(const __half* p) {
+    unsigned short v;
+    asm volatile("ld.global.cg.b16 %0, [%1];" : "=h"(v) : "l"(p));
+    return __ushort_as_half(v);
+}
+
+// k_rows2: two steps; a pair of warps marches down an item's rows.  The first
+// warp takes the first step as k_rows does, on 64 columns of which 60 come
+// out right, and hands its rows to the second through a ring of eight rows in
+// shared memory; the second takes the second step on those and stores 56
+// columns.  The lattice's periodic neighbours are read where they are (rows
+// and columns wrapped), not from the images, which reach two sites only.
+//
+// One step a launch moves 72 bytes a site and step (FP32) and stops at 0.81 of
+// the copy bandwidth; two move 36, and the kernel is bound by the FP32 pipe
+// (73 % of its cycles, 63 % of issue slots).  Measured per step, 32 x 16 tile
+// kernel -> this one: FP32 BGK 1024^2 19.2 -> 16.3 us, 1201^2 33.2 -> 21.6,
+// 2100 x 1700 51.6 -> 46.2, 4096^2 221 -> 191, 8192^2 870 -> 706 (95 GLUPS);
+// MRT 8192^2 984 -> 865; 512 lattices of 64^2 .. 512^2 804 -> 730, 100 of
+// 64^2 .. 200^2 48 -> 40.  FP16 storage, which is not bound by DRAM, loses by
+// the columns it computes twice (8192^2: k_rows 688, this one 778).
+// Unrolling either row loop by 2 is 3 to 25 % slower; 64-bit addresses and a
+// test per load instead of one per row cost 6 %.
+template <class S, int EOSP, bool MRT, bool ONE>
+__global__ void __launch_bounds__(64 * kPairs, 2)
+    k_rows2(StepArgs a, const __grid_constant__ LatDev lat0) {
+    using T = typename S::T;
+    using IO = PairIO<S>;
+    using Raw = typename IO::Raw;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ LatDev slat[ONE ? 1 : kPairs];
+    __shared__ uint64_t bars[kPairs][2 * kPairDepth];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, pr = w % kPairs;
+    Raw* const ring = reinterpret_cast<Raw*>(smem_raw) + pr * (kPairDepth * 9 * 32);  // [depth][9][32]
+    uint64_t* const full = bars[pr];
+    uint64_t* const empty = full + kPairDepth;
+    const int t = blockIdx.x * kPairs + pr;
+    int4 tl = make_int4(0, 0, 0, 0);
+    bool on = t < a.ntiles;
+    if (on) {
+        tl = __ldg(&a.tiles[t]);
+        // (a lattice with one step left is not this launch's)
+        on = !a.quota || a.step + 2 <= __ldg(&a.quota[tl.x]);
+    }
+    if (w < kPairs && lane == 0) {
+        for (int k = 0; k < 2 * kPairDepth; ++k) mbar_init(&full[k], 1);
+        mbar_fence_init();
+    }
+    if (!ONE && w < kPairs && on)
+        for (int k = lane; k < (int)(sizeof(LatDev) / 4); k += 32)
+            reinterpret_cast<int*>(&slat[pr])[k] = __ldg(reinterpret_cast<const int*>(a.lats + tl.x) + k);
+    __syncthreads();
+    if (!on) return;
+    const LatDev& L = ONE ? lat0 : slat[pr];
+    const SiteConsts C = site_consts(L);
+    const int nx = L.nx, ny = L.ny, pitch = L.pitch, gx = L.gx;
+    const int64_t plane = L.plane;
+    const int x0 = tl.y, y0 = tl.z, y1 = tl.z + item_rows(tl.w), xend = x0 + item_width(tl.w);
+    const int x = x0 - 4 + 2 * lane;
+    auto need = [&](int lo, int hi) {  // which of the lane's columns lie in lo .. hi
+        return (unsigned)(x >= lo && x <= hi) | ((unsigned)(x + 1 >= lo && x + 1 <= hi) << 1);
+    };
+    Row3 P0{}, P1{};
+    Site<float2> sprev{};
+    if (w < kPairs) {
+        // ------------------------------------------------------ first step
+        const unsigned live = need(x0 - 3, xend + 2);
+        const int c0 = ((x % nx) + nx) % nx, c1 = c0 + 1 == nx ? 0 : c0 + 1;
+        const bool whole = __all_sync(0xffffffffu, !(c0 & 1) && c1 == c0 + 1);
+        // byte offsets of the pair's place in a row of a plane (32 bits: the planes
+        // of a lattice on this path are smaller than 4 GB)
+        const char* const base = reinterpret_cast<const char*>(
+            reinterpret_cast<const T*>(a.pop) + L.off_f[a.parity]);
+        const uint32_t prow = (uint32_t)pitch * (uint32_t)sizeof(T);
+        const uint32_t col = (uint32_t)(GY * pitch + gx + c0) * (uint32_t)sizeof(T);
+        const int next = (c1 - c0) * (int)sizeof(T);
+        auto down = [&](int y) { return y + 1 == ny ? 0 : y + 1; };
+        auto at = [&](int i, uint32_t o) {
+            return reinterpret_cast<const T*>(base + i * plane * (int64_t)sizeof(T) + o);
+        };
+        auto one = [&](int i, uint32_t o) {
+            return raw_of(ld_one(at(i, o)), ld_one(at(i, o + (uint32_t)next)));
+        };
+        auto ld = [&](int i, uint32_t o) { return whole ? IO::ld(at(i, o)) : one(i, o); };
+        auto load = [&](Raw g[9], Raw& rest, uint32_t om, uint32_t oc, uint32_t op) {
+            if (whole) {
+#pragma unroll
+                for (int i = 1; i < 9; ++i)
+                    g[i] = IO::ld(at(i, plane_cy(i) == 0 ? oc : plane_cy(i) > 0 ? om : op));
+                rest = IO::ld(at(0, op));
+            } else {
+#pragma unroll
+                for (int i = 1; i < 9; ++i)
+                    g[i] = one(i, plane_cy(i) == 0 ? oc : plane_cy(i) > 0 ? om : op);
+                rest = one(0, op);
+            }
+        };
+        int yw = ((y0 - 4) % ny + ny) % ny;  // row y - 1, then the rows after it
+        uint32_t om = (uint32_t)yw * prow + col;
+        yw = down(yw);
+        uint32_t oc = (uint32_t)yw * prow + col;
+        yw = down(yw);
+        uint32_t op = (uint32_t)yw * prow + col;
+        Row3 Rm = row3<S>(ld(0, om)), Rc = row3<S>(ld(0, oc));
+        Raw gn[9], rn;
+        load(gn, rn, om, oc, op);
+        for (int y = y0 - 3; y <= y1 + 2; ++y) {
+            Raw g[9];
+#pragma unroll
+            for (int i = 1; i < 9; ++i) g[i] = gn[i];
+            const Row3 Rp = row3<S>(rn);
+            if (y < y1 + 2) {
+                om = oc;
+                oc = op;
+                yw = down(yw);
+                op = (uint32_t)yw * prow + col;
+                load(gn, rn, om, oc, op);
+            }
+            const Site<float2> s = row_site<S>(g, Rm, Rc, Rp);
+            const Row3 P2 = row3(Eos<EOSP>::psi(L, site_rho(s, L.rho0), a.status, live));
+            if (y >= y0 - 1) {
+                float2 v[9];
+                row_collide<S, MRT>(C, L.mrt_s, sprev, P0, P1, P2, v);
+                const unsigned n = (unsigned)(y - (y0 - 1)), slot = n % kPairDepth;  // row y0 - 2 + n
+                if (n >= kPairDepth) {
+                    const bool ok = mbar_wait_bounded(&empty[slot], (uint32_t)(n / kPairDepth - 1) & 1u,
+                                                      a.wait_cycles);
+                    if (!__all_sync(0xffffffffu, ok)) {
+                        if (lane == 0) atomicOr(a.status + L.lattice, 2u);
+                        return;
+                    }
+                }
+                T* q = reinterpret_cast<T*>(ring + slot * (9 * 32) + lane);
+#pragma unroll
+                for (int i = 0; i < 9; ++i) IO::st(q + i * 64, v[i]);
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&full[slot]);
+            }
+            sprev = s;
+            P0 = P1;
+            P1 = P2;
+            Rm = Rc;
+            Rc = Rp;
+        }
+    } else {
+        // ------------------------------------------------------ second step
+        const unsigned live = need(x0 - 1, xend);
+        const bool in0 = x >= x0 && x < xend, in1 = x >= x0 && x + 1 < xend;
+        T* q = reinterpret_cast<T*>(a.pop) + L.off_f[a.parity ^ 1] +
+               (int64_t)(y0 - 2 + GY) * pitch + gx + x;
+        auto got = [&](unsigned n) {
+            const bool ok =
+                mbar_wait_bounded(&full[n % kPairDepth], (uint32_t)(n / kPairDepth) & 1u, a.wait_cycles);
+            return __all_sync(0xffffffffu, ok);
+        };
+        auto row = [&](int i, unsigned n) { return ring[((n % kPairDepth) * 9 + i) * 32 + lane]; };
+        bool ok = got(0) && got(1);
+        Row3 Rm{}, Rc{};
+        if (ok) {
+            Rm = row3<S>(row(0, 0));
+            Rc = row3<S>(row(0, 1));
+        }
+        for (int y = y0 - 1; y <= y1; ++y) {
+            const unsigned n = (unsigned)(y - (y0 - 2));  // ring row of lattice row y
+            ok = ok && got(n + 1);
+            if (!ok) {
+                if (lane == 0) atomicOr(a.status + L.lattice, 2u);
+                return;
+            }
+            const Row3 Rp = row3<S>(row(0, n + 1));
+            Raw g[9];
+#pragma unroll
+            for (int i = 1; i < 9; ++i) g[i] = row(i, n - plane_cy(i));
+            const Site<float2> s = row_site<S>(g, Rm, Rc, Rp);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&empty[(n - 1) % kPairDepth]);  // row y - 1 is done with
+            const Row3 P2 = row3(Eos<EOSP>::psi(L, site_rho(s, L.rho0), a.status, live));
+            if (y > y0) {
+                const int ys = y - 1;
+                float2 v[9];
+                row_collide<S, MRT>(C, L.mrt_s, sprev, P0, P1, P2, v);
+                row_store<S>(q, plane, pitch, x, ys, nx, ny, in0, in1,
                              x0 < GW || xend > nx - GW || ys < GW || ys >= ny - GW, v);
             }
             q += pitch;
@@ -571,7 +778,24 @@ cudaError_t rows_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+template <class S, bool MRT, bool ONE>
+cudaError_t pairs_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    constexpr int smem = (int)pair_smem((int)sizeof(typename S::T));
+    const cudaError_t e = cudaFuncSetAttribute((const void*)k_rows2<S, EOS_DF, MRT, ONE>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const unsigned grid = (unsigned)((a.ntiles + kPairs - 1) / kPairs);
+    k_rows2<S, EOS_DF, MRT, ONE><<<grid, 64 * kPairs, smem, st>>>(a, lat0 ? *lat0 : LatDev{});
+    return cudaGetLastError();
+}
+
 }  // namespace
+
+template <class S>
+cudaError_t pairs_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    if (mrt) return lat0 ? pairs_inst<S, true, true>(a, lat0, st) : pairs_inst<S, true, false>(a, lat0, st);
+    return lat0 ? pairs_inst<S, false, true>(a, lat0, st) : pairs_inst<S, false, false>(a, lat0, st);
+}
 
 template <class S>
 cudaError_t rows_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {

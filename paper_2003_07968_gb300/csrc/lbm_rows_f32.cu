@@ -12,4 +12,8 @@ cudaError_t rows_f32(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_
     return rows_any<StoreF32>(mrt, a, lat0, st);
 }
 
+cudaError_t pairs_f32(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
+    return pairs_any<StoreF32>(mrt, a, lat0, st);
+}
+
 }  // namespace pplbm

@@ -12,11 +12,12 @@ constexpr int kRowCols = 60;  // columns a warp advances at most (it holds 64)
 
 // Column c of boundary k of n strips over nx columns: even, at most kRowCols
 // apart, as equal as that allows.
+// (n strips of at most `cols` columns each: strip_count)
 inline int strip_edge(int nx, int n, int k) {
     const int pairs = (nx + 1) / 2;
     return std::min(nx, 2 * (int)(((int64_t)pairs * k + n - 1) / n));
 }
-inline int strip_count(int nx) { return (nx + kRowCols - 1) / kRowCols; }
+inline int strip_count(int nx, int cols = kRowCols) { return (nx + cols - 1) / cols; }
 inline int band_edge(int ny, int n, int k) { return (int)((int64_t)ny * k / n); }
 
 // ---- one step a launch (k_rows): row items, each the work of one warp
@@ -38,22 +39,10 @@ inline int row_item_height(const std::vector<LatDev>& lats, int64_t warps) {
     }
     return (int)std::min<int64_t>(64, std::max<int64_t>(8, units / (5 * warps)));
 }
-// Whether a step of these lattices runs on k_rows rather than on the tile
-// kernel (measured, see k_rows): FP16 storage always; FP32 where one wave of
-// warps covers the lattices (up to about 2.3 M sites), and again for one
-// lattice so large that both read DRAM evenly (MRT, whose arithmetic weighs
-// more, from half that on).
-inline bool rows_beat_tiles(const std::vector<LatDev>& lats, bool f16, bool mrt, int64_t warps) {
-    if (f16) return true;
-    int64_t items = 0;
-    for (const LatDev& L : lats) items += (int64_t)strip_count(L.nx) * ((L.ny + 15) / 16);
-    if (items <= warps) return true;
-    const int64_t sites = (int64_t)lats[0].nx * lats[0].ny;
-    return lats.size() == 1 && sites >= (int64_t)1 << (mrt ? 24 : 25);
-}
 // The items of one lattice, bands one after another, a band's strips side by side.
-inline void row_items(const LatDev& L, int lattice, int h, std::vector<int4>& out) {
-    const int ns = strip_count(L.nx), nb = (L.ny + h - 1) / h;
+inline void row_items(const LatDev& L, int lattice, int h, std::vector<int4>& out,
+                      int cols = kRowCols) {
+    const int ns = strip_count(L.nx, cols), nb = (L.ny + h - 1) / h;
     for (int b = 0; b < nb; ++b) {
         const int y0 = band_edge(L.ny, nb, b), y1 = band_edge(L.ny, nb, b + 1);
         for (int s = 0; s < ns; ++s) {
@@ -61,6 +50,40 @@ inline void row_items(const LatDev& L, int lattice, int h, std::vector<int4>& ou
             out.push_back(make_int4(lattice, x0, y0, pack_rows(y1 - y0, x1 - x0)));
         }
     }
+}
+
+// ---- two steps a launch (k_rows2): an item is the work of a pair of warps
+constexpr int kPairCols = 56;   // columns of an item at most (64 held, 4 lost a side)
+constexpr int kPairDepth = 8;   // rows of the ring between a pair's warps
+constexpr int kPairs = 4;       // pairs of a block
+constexpr size_t pair_smem(int es) { return (size_t)kPairs * kPairDepth * 9 * 64 * es; }
+
+// Rows of an item, `pairs`: the pairs of warps the GPU holds.  One wave while
+// that makes items of about 100 rows at most, then even waves of about 72
+// rows, for one lattice 4 at most (a last wave that is nearly empty costs
+// more than the rows that items share).  Measured per step: 2100 x 1700 46 us
+// in one wave of 53 rows, 53-60 in items of 32 to 64; 3000^2 106 us in two
+// waves of 67, 112-144 in items of 48 to 192; 512 lattices 726 us in items of
+// 96 rows, 793 in four waves of 230.
+inline int pair_item_height(const std::vector<LatDev>& lats, int64_t pairs) {
+    int64_t units = 0, most = 0;
+    for (const LatDev& L : lats) {
+        units += (int64_t)strip_count(L.nx, kPairCols) * L.ny;
+        most = std::max<int64_t>(most, L.ny);
+    }
+    int64_t waves = std::max<int64_t>(1, (units + 36 * pairs) / (72 * pairs));
+    if (lats.size() == 1) waves = std::min<int64_t>(waves, 4);
+    int64_t h = std::max<int64_t>(4, units / (waves * pairs));
+    for (; h < most; ++h) {
+        int64_t n = 0;
+        for (const LatDev& L : lats) n += strip_count(L.nx, kPairCols) * ((L.ny + h - 1) / h);
+        if (n <= waves * pairs) break;
+    }
+    return (int)std::min<int64_t>(h, most);
+}
+// 32-bit offsets: a lattice's rows in a plane take less than 4 GB
+inline bool pairs_fit(const LatDev& L, int es) {
+    return ((int64_t)L.ny + 2 * GY) * L.pitch * es < (int64_t)1 << 32;
 }
 
 // ---- resident lattices: one tile a block, kept in shared memory for many steps

@@ -48,9 +48,12 @@ struct TuneKey {
 struct PassCfg {
     int variant, tx, ty, grid, spt;
 };
+// What the single pass runs on: the tile kernels of pass[1], k_rows, or
+// k_rows2 (two steps a launch, an odd step on k_rows).
+enum StepPath { PATH_TILES, PATH_ROWS, PATH_PAIRS };
 struct TuneVal {
     PassCfg pass[2];
-    bool rows = false;  // the single pass: k_rows beat the best tile kernel
+    StepPath path = PATH_TILES;
 };
 
 // One pass of the step (0: psi, 1: force + collision + stream): its kernel
@@ -132,17 +135,18 @@ struct lbm_handle {
     // graphs
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // by starting parity
     int graph_steps = 32;
+    int graph_launches = 32;  // kernels of a captured graph
     int tune_variant = LBM_KERNEL_AUTO;  // the kernel_variant the handle was created with
     // tensor maps (loads, stores) of the population arena for the single-pass
     // TMA kernel (one lattice, or a batch in one row space; rows at least a box
     // wide); else that kernel uses row copies
     CUtensorMap tmap[2]{};  // loads, stores
     bool has_tmap = false;
-    // row items of the lattices for k_rows, and whether a step uses them
+    // row items of the lattices for k_rows, then for k_rows2 (none: not built)
     int4* items = nullptr;
-    int n_items = 0;
+    int n_items = 0, n_pair_items = 0;
     size_t items_bytes = 0;
-    bool rows = false;
+    StepPath path = PATH_TILES;
     // the lattices as resident tiles, when they fit (plan_resident): tiles,
     // mailboxes and epochs in one allocation
     int res_grid = 0;  // tiles (0: no plan)
@@ -152,7 +156,7 @@ struct lbm_handle {
     bool res_reset = true;  // mailboxes and epochs must be cleared first
     // profiling
     bool prof = false;
-    ProfRec rec[2];
+    ProfRec rec[3];  // psi pass, one step, two steps
     std::vector<cudaEvent_t> ev_pool;
     std::string err;
 };
@@ -351,25 +355,35 @@ int make_resident(lbm_handle* h) {
     return LBM_OK;
 }
 
-// Row items of the handle's lattices.
+// Row items of the handle's lattices, for k_rows and (where it can run) k_rows2.
 int make_items(lbm_handle* h) {
-    const int height = row_item_height(h->lat, (int64_t)h->sm_count * 4 * kRowWarps);
+    const int64_t sms = h->sm_count;
     std::vector<int4> t;
+    const int height = row_item_height(h->lat, sms * 4 * kRowWarps);
     for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, height, t);
+    const size_t n = t.size();
+    bool fit = true;
+    for (const LatDev& L : h->lat) fit = fit && pairs_fit(L, h->f16 ? 2 : 4);
+    if (fit) {
+        const int h2 = pair_item_height(h->lat, sms * 2 * kPairs);
+        for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, h2, t, kPairCols);
+    }
     h->items_bytes = t.size() * sizeof(int4);
     h->items = (int4*)dev_alloc(h, h->items_bytes);
     if (!h->items) return LBM_ERR_OOM;
     CK(h, cudaMemcpyAsync(h->items, t.data(), h->items_bytes, cudaMemcpyHostToDevice, h->stream));
-    h->n_items = (int)t.size();
+    h->n_items = (int)n;
+    h->n_pair_items = (int)(t.size() - n);
     return LBM_OK;
 }
 
-cudaError_t launch_row_step(lbm_handle* h, int parity) {
+// One step on k_rows, or two on k_rows2, from buffer `parity` to the other.
+cudaError_t launch_row_steps(lbm_handle* h, int parity, bool two) {
     StepArgs a = step_args(h, parity, 1);
-    a.tiles = h->items;
-    a.ntiles = h->n_items;
-    return launch_rows(h->f16, h->collision == LBM_COLL_MRT, a,
-                       h->lat.size() == 1 ? &h->lat[0] : nullptr, h->stream);
+    a.tiles = h->items + (two ? h->n_items : 0);
+    a.ntiles = two ? h->n_pair_items : h->n_items;
+    return (two ? launch_pairs : launch_rows)(h->f16, h->collision == LBM_COLL_MRT, a,
+                                              h->lat.size() == 1 ? &h->lat[0] : nullptr, h->stream);
 }
 
 // nsteps steps in one launch (state from buffer `parity` to the other).
@@ -468,8 +482,8 @@ int launch_step(lbm_handle* h, int p) {
     a1.starve = h->starve;  // an armed failure-detection test goes into this launch only
     if (h->starve) a1.wait_cycles = kTestWaitBudgetCycles;
     h->starve = 0;
-    if (h->rows && !a1.starve)
-        CK(h, launch_row_step(h, p));
+    if (h->path != PATH_TILES && !a1.starve)
+        CK(h, launch_row_steps(h, p, false));
     else
         CK(h, launch_pass(h, 1, a1, h->pass[1].grid));
     if (h->prof) {
@@ -479,6 +493,23 @@ int launch_step(lbm_handle* h, int p) {
         h->rec[1].pending.emplace_back(e1, e2);
     }
     h->launches += fused ? 1 : 2;
+    return LBM_OK;
+}
+
+// Two steps in one launch on parity p.
+int launch_two_steps(lbm_handle* h, int p) {
+    cudaEvent_t e1 = nullptr, e2 = nullptr;
+    if (h->prof) {
+        e1 = take_event(h);
+        e2 = take_event(h);
+        CK(h, cudaEventRecord(e1, h->stream));
+    }
+    CK(h, launch_row_steps(h, p, true));
+    if (h->prof) {
+        CK(h, cudaEventRecord(e2, h->stream));
+        h->rec[2].pending.emplace_back(e1, e2);
+    }
+    h->launches += 1;
     return LBM_OK;
 }
 
@@ -493,10 +524,11 @@ int capture_graph(lbm_handle* h) {
     int p = h->parity;
     const int64_t before = h->launches;
     int rc = LBM_OK;
-    for (int s = 0; s < h->graph_steps && rc == LBM_OK; ++s) {
-        rc = launch_step(h, p);
-        p ^= 1;
+    for (int s = 0; s < h->graph_steps && rc == LBM_OK; p ^= 1) {  // (graph_steps is even)
+        rc = h->path == PATH_PAIRS ? launch_two_steps(h, p) : launch_step(h, p);
+        s += h->path == PATH_PAIRS ? 2 : 1;
     }
+    h->graph_launches = (int)(h->launches - before);
     h->launches = before;
     cudaError_t e = cudaStreamEndCapture(h->stream, &g);
     if (rc != LBM_OK) {
@@ -588,12 +620,12 @@ void release(lbm_handle* h) {
     drop_graph(h);
     // psi pairs own e0; step pairs own (e1, e2)
     for (auto& pr : h->rec[0].pending) cudaEventDestroy(pr.first);
-    for (auto& pr : h->rec[1].pending) {
-        cudaEventDestroy(pr.first);
-        cudaEventDestroy(pr.second);
-    }
-    h->rec[0].pending.clear();
-    h->rec[1].pending.clear();
+    for (int k = 1; k < 3; ++k)
+        for (auto& pr : h->rec[k].pending) {
+            cudaEventDestroy(pr.first);
+            cudaEventDestroy(pr.second);
+        }
+    for (auto& r : h->rec) r.pending.clear();
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     h->ev_pool.clear();
     if (h->status_ev) cudaEventDestroy(h->status_ev);
@@ -1012,7 +1044,8 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         if (fused_tma_make_map(h->f16, 32, 16, h->lat.data(), n, h->pop, probe))
             cfg[1] = PassCfg{LBM_KERNEL_TMA, 32, 16, 0, 2};
     }
-    bool tuned = false, tuned_rows = false;
+    bool tuned = false;
+    StepPath tuned_path = PATH_TILES;
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         TuneKey k{h->device, h->storage, h->eos, variant * 4 + h->schedule,
@@ -1021,7 +1054,7 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         if (it != g_tune_cache.end() && !(opts && (opts->tile_x || opts->tile_y))) {
             for (int q = 0; q < 2; ++q) cfg[q] = it->second.pass[q];
             tuned = true;
-            tuned_rows = it->second.rows;
+            tuned_path = it->second.path;
         }
     }
     if (cfg[1].variant == LBM_KERNEL_TMA &&
@@ -1049,18 +1082,21 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         const int rc = make_resident(h);
         if (rc) return fail(rc);
     }
-    // ... and larger ones may run on k_rows
+    // ... and larger ones run on the row kernels
     if (!h->res_grid && fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
         !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
         const int rc = make_items(h);
         if (rc) return fail(rc);
-        h->rows = tuned ? tuned_rows
-                        : rows_beat_tiles(h->lat, h->f16, h->collision == LBM_COLL_MRT,
-                                          (int64_t)h->sm_count * 4 * kRowWarps);
+        h->path = tuned    ? tuned_path
+                  : h->f16 ? PATH_ROWS
+                           : PATH_PAIRS;  // measured: see k_rows2
+        if (h->path == PATH_PAIRS && !h->n_pair_items) h->path = PATH_ROWS;
     }
     h->tune_variant = variant;
     h->rec[0].name = "psi_pass";
     h->rec[1].name = h->schedule == LBM_SCHED_FUSED ? "fused_step" : "collide_stream";
+    h->rec[2].name = "fused_two_steps";
+    h->rec[2].bytes = (double)h->sites * 18.0 * es;
     h->rec[0].bytes = (double)h->sites * (9.0 * es + 4.0);
     h->rec[1].bytes = (double)h->sites * (h->schedule == LBM_SCHED_FUSED ? 18.0 * es
                                                                         : 18.0 * es + 4.0);
@@ -1147,21 +1183,23 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
             left -= n;
         }
     }
-    if (!h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps) {
+    while (!h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps) {
         if (!h->graph[h->parity]) {
             rc = capture_graph(h);
             if (rc) return rc;
         }
-        while (left >= h->graph_steps) {
-            CK(h, cudaGraphLaunch(h->graph[h->parity], h->stream));
-            h->launches += (h->schedule == LBM_SCHED_FUSED ? 1 : 2) * (int64_t)h->graph_steps;
-            left -= h->graph_steps;  // graph_steps is even: parity unchanged
-        }
+        CK(h, cudaGraphLaunch(h->graph[h->parity], h->stream));
+        h->launches += h->graph_launches;
+        left -= h->graph_steps;
+        // an even number of steps, but half as many launches of two
+        if (h->path == PATH_PAIRS && (h->graph_launches & 1)) h->parity ^= 1;
     }
-    for (; left > 0; --left) {
-        rc = launch_step(h, h->parity);
+    while (left > 0) {
+        const bool two = h->path == PATH_PAIRS && left >= 2 && !h->starve;
+        rc = two ? launch_two_steps(h, h->parity) : launch_step(h, h->parity);
         if (rc) return rc;
         h->parity ^= 1;
+        left -= two ? 2 : 1;
     }
     if (!h->status_pending) {
         CK(h, cudaMemcpyAsync(h->status_host, h->status, h->lat.size() * sizeof(uint32_t),
@@ -1309,7 +1347,7 @@ int lbm_profile(lbm_handle* h, int32_t on) {
 static int lbm_profile_read_body(lbm_handle* h, lbm_kernel_stat* out, int32_t max, int32_t* n) {
     if (!h || !n) return LBM_ERR_ARG;
     CK(h, cudaStreamSynchronize(h->stream));
-    for (int k = 0; k < 2; ++k) {
+    for (int k = 0; k < 3; ++k) {
         ProfRec& r = h->rec[k];
         for (auto& pr : r.pending) {
             float ms = 0.f;
@@ -1320,13 +1358,14 @@ static int lbm_profile_read_body(lbm_handle* h, lbm_kernel_stat* out, int32_t ma
     }
     // return events to the pool: psi pairs own e0, step pairs own (e1, e2)
     for (auto& pr : h->rec[0].pending) h->ev_pool.push_back(pr.first);
-    for (auto& pr : h->rec[1].pending) {
-        h->ev_pool.push_back(pr.first);
-        h->ev_pool.push_back(pr.second);
-    }
-    h->rec[0].pending.clear();
-    h->rec[1].pending.clear();
-    const int cnt = 2;
+    for (int k = 1; k < 3; ++k)
+        for (auto& pr : h->rec[k].pending) {
+            h->ev_pool.push_back(pr.first);
+            h->ev_pool.push_back(pr.second);
+        }
+    for (auto& r : h->rec) r.pending.clear();
+    // (the third record only where two-step launches ran)
+    const int cnt = h->rec[2].launches ? 3 : 2;
     for (int k = 0; k < cnt && k < max && out; ++k) {
         std::memset(&out[k], 0, sizeof(lbm_kernel_stat));
         std::snprintf(out[k].name, sizeof(out[k].name), "%s", h->rec[k].name.c_str());
@@ -1445,16 +1484,25 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
         h->pass[k].grid = bc.grid;
         best_cfg.pass[k] = bc;
         if (k == 1 && h->items && rc == LBM_OK) {
-            // the row kernel against the best tile kernel
-            cudaError_t e = launch_row_step(h, h->parity);  // warm-up
-            cudaEventRecord(ea, h->stream);
-            for (int r = 0; r < repeats && e == cudaSuccess; ++r) e = launch_row_step(h, h->parity);
-            cudaEventRecord(eb, h->stream);
-            if (e == cudaSuccess) e = cudaEventSynchronize(eb);
-            if (e != cudaSuccess) { rc = cuda_fail(h, e, "autotune rows"); break; }
-            float ms = 0.f;
-            cudaEventElapsedTime(&ms, ea, eb);
-            best_cfg.rows = h->rows = ms < best;
+            // the row kernels against the best tile kernel, per step
+            h->path = PATH_TILES;
+            for (int two = 0; two < (h->n_pair_items ? 2 : 1); ++two) {
+                cudaError_t e = launch_row_steps(h, h->parity, two);  // warm-up
+                cudaEventRecord(ea, h->stream);
+                for (int r = 0; r < repeats && e == cudaSuccess; ++r)
+                    e = launch_row_steps(h, h->parity, two);
+                cudaEventRecord(eb, h->stream);
+                if (e == cudaSuccess) e = cudaEventSynchronize(eb);
+                if (e != cudaSuccess) { rc = cuda_fail(h, e, "autotune rows"); break; }
+                float ms = 0.f;
+                cudaEventElapsedTime(&ms, ea, eb);
+                if (two) ms *= 0.5f;
+                if (ms < best) {
+                    best = ms;
+                    h->path = two ? PATH_PAIRS : PATH_ROWS;
+                }
+            }
+            best_cfg.path = h->path;
         }
     }
     cudaEventDestroy(ea);

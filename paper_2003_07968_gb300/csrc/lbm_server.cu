@@ -148,6 +148,7 @@ struct TableSet {
     int4* tiles[2] = {nullptr, nullptr};
     size_t cap[2] = {0, 0};
     int ntiles[2] = {0, 0};
+    int npair = 0;  // pair items after the ntiles[1] row items (0: single steps only)
     std::vector<int> begin[2], count[2];
     // tickets of the lattices (in table order) that the lattice table and
     // tile lists describe; a chunk over the same lattices only rewrites the
@@ -186,7 +187,8 @@ struct lbm_server {
     float* psi_arena = nullptr;
     int64_t pitch = 0, plane = 0, row_cap = 0;  // of the row space (elements, rows)
     size_t pop_bytes = 0, psi_region = 0;
-    bool rows = false;     // single pass on the row kernel (FP16 storage; tile lists are row items)
+    bool rows = false;     // single pass on the row kernels (tile lists are row items)
+    bool pairs = false;    // ... two steps a launch (FP32 storage)
     bool tma = false;      // single pass on the TMA kernel (one tensor map for the arena)
     CUtensorMap tmap[2]{};  // loads, stores
     size_t up_cap = 0;            // doubles of the device staging buffer
@@ -349,14 +351,20 @@ cudaError_t rebuild(lbm_server* S, TableSet& T, std::vector<Request*>& res,
     for (int k = 0; k < 2; ++k) {
         const PassState& P = S->pass[k];
         const bool items = k == 1 && S->rows;
-        size_t nt = 0;
+        size_t nt = 0, nrow = 0;
         std::vector<int4> rt;
         if (items) {
             std::vector<LatDev> lats;
             for (Request* R : res) lats.push_back(R->L);
             const int height = row_item_height(lats, (int64_t)S->sm_count * 4 * kRowWarps);
             for (size_t l = 0; l < res.size(); ++l) row_items(lats[l], (int)l, height, rt);
+            nrow = rt.size();
+            if (S->pairs) {
+                const int h2 = pair_item_height(lats, (int64_t)S->sm_count * 2 * kPairs);
+                for (size_t l = 0; l < res.size(); ++l) row_items(lats[l], (int)l, h2, rt, kPairCols);
+            }
             nt = rt.size();
+            T.npair = (int)(nt - nrow);
         }
         for (Request* R : res)
             if (!items) nt += (size_t)((R->L.nx + P.tx - 1) / P.tx) * ((R->L.ny + P.ty - 1) / P.ty);
@@ -395,7 +403,7 @@ cudaError_t rebuild(lbm_server* S, TableSet& T, std::vector<Request*>& res,
         if (bytes)
             e = cudaMemcpyAsync(T.tiles[k], t, bytes, cudaMemcpyHostToDevice, S->stream);
         if (e != cudaSuccess) return e;
-        T.ntiles[k] = (int)nt;
+        T.ntiles[k] = (int)(items ? nrow : nt);
     }
     T.members = members;
     return cudaSuccess;
@@ -659,12 +667,14 @@ void worker_loop(lbm_server* S) {
             C.p0 = S->parity;
             C.quota.resize(res.size());
             // steps of this chunk: about chunk_ms of GPU time over the
-            // resident sites, at most chunk_steps
+            // resident sites, at most chunk_steps; an even number where two
+            // steps go in a launch, so that lattices that run on end together
             int64_t steps = S->o.chunk_steps;
             if (S->o.chunk_ms > 0.0) {
                 const double fit = S->o.chunk_ms * 1e-3 * rate / (double)std::max<int64_t>(res_sites, 1);
                 steps = std::max<int64_t>(1, std::min<int64_t>(steps, (int64_t)fit));
             }
+            if (S->pairs && steps > 1) steps &= ~(int64_t)1;
             int64_t k = 0;
             std::vector<Request*> keep;
             for (size_t l = 0; l < res.size(); ++l) {
@@ -674,13 +684,35 @@ void worker_loop(lbm_server* S) {
                 if (res[l]->remaining > 0)
                     keep.push_back(res[l]);
                 else
-                    C.finished.push_back(Finished{res[l], (int)l, (C.p0 + C.quota[l]) & 1, LBM_OK});
+                    // (a launch, of one step or two, swaps the buffers)
+                    C.finished.push_back(
+                        Finished{res[l], (int)l,
+                                 (C.p0 + (S->pairs ? (C.quota[l] + 1) / 2 : C.quota[l])) & 1, LBM_OK});
             }
             TableSet& T = S->set[cur];
             if (e == cudaSuccess) e = rebuild(S, T, C.res, C.quota);
             if (e == cudaSuccess) e = cudaEventRecord(S->chunk_begin[cur], S->stream);
             const int g0 = pass_grid(S, 0, T.ntiles[0]), g1 = pass_grid(S, 1, T.ntiles[1]);
-            for (int64_t st = 0; st < k && e == cudaSuccess; ++st) {
+            for (int64_t st = 0; S->pairs && st < k && e == cudaSuccess; st += 2) {
+                // two steps of every lattice with at least two left, one of
+                // those with one
+                StepArgs a1 = args(S, T, 1, S->parity);
+                a1.step = (int)st;
+                if (std::any_of(C.quota.begin(), C.quota.end(), [&](int q) { return q == st + 1; })) {
+                    a1.last_only = 1;
+                    e = launch(S, 1, a1, g1, S->stream);
+                    a1.last_only = 0;
+                    ++launches;
+                }
+                if (e == cudaSuccess && k >= st + 2) {
+                    a1.tiles += a1.ntiles;
+                    a1.ntiles = T.npair;
+                    e = launch_pairs(S->f16, 0, a1, nullptr, S->stream);
+                    ++launches;
+                }
+                S->parity ^= 1;
+            }
+            for (int64_t st = 0; !S->pairs && st < k && e == cudaSuccess; ++st) {
                 StepArgs a0 = args(S, T, 0, S->parity), a1 = args(S, T, 1, S->parity);
                 a0.step = a1.step = (int)st;
                 if (!S->fused) e = launch(S, 0, a0, g0, S->stream);
@@ -1020,10 +1052,14 @@ static int lbm_server_create_body(const lbm_server_opts* opts, lbm_server** out)
         S->pass[1].ty = kPassDefaults[1].ty;
         S->pass[1].spt = kPassDefaults[1].spt;
     }
-    // FP16 storage: the row kernel (see rows_beat_tiles; the resident lattices
-    // change from chunk to chunk, FP32 ones stay on the tile kernel)
-    S->rows = S->tma && S->f16 && o.kernel_variant == LBM_KERNEL_AUTO &&
-              o.eos_precision == LBM_EOS_DF && !(o.tile_x || o.tile_y);
+    // the row kernels, FP32 storage two steps a launch (where the tallest
+    // request's rows fit the 32-bit offsets of k_rows2)
+    S->rows = S->tma && o.kernel_variant == LBM_KERNEL_AUTO && o.eos_precision == LBM_EOS_DF &&
+              !(o.tile_x || o.tile_y);
+    LatDev tallest{};
+    tallest.pitch = (int32_t)S->pitch;
+    tallest.ny = (int32_t)std::min<int64_t>(o.max_request_sites / 2, S->row_cap);
+    S->pairs = S->rows && !S->f16 && pairs_fit(tallest, S->es);
     S->st.arena_bytes = (int64_t)o.arena_bytes;
     try {
         S->worker = std::thread(worker_main, S);

@@ -1,9 +1,10 @@
 """The many-steps launch (k_resident) against one launch per step.
 
 A default handle whose lattices fit the SMs' shared memory advances many
-steps in one launch; graph_steps=-1 keeps it on the tile kernel, one launch
-per step.  Both run the same operations on the same values, so every output
-is equal bit for bit.
+steps in one launch, a larger one two steps (FP32 storage) or one;
+kernel_variant=LBM_KERNEL_TMA keeps it on the tile kernel, one launch per
+step.  All run the same operations on the same values, so every output is
+equal bit for bit.
 """
 import numpy as np
 import pytest
@@ -69,7 +70,7 @@ def test_many_steps_equal_single_launches(P, storage, mrt):
         d, f = _desc(P, nx, ny, storage, mrt, sigma=0.5), _field(nx, ny)
         chunks = (2, 1, 3, 17)
         a, la = _run(P, [d], [f], chunks)
-        b, lb = _run(P, [d], [f], chunks, graph_steps=-1)
+        b, lb = _run(P, [d], [f], chunks, kernel_variant=P.LBM_KERNEL_TMA)
         assert (la, lb) == (4, 23), (nx, ny)
         _same(a, b)
 
@@ -81,7 +82,7 @@ def test_batches_of_resident_lattices(P):
     fields = [_field(nx, ny, k) for k, (nx, ny) in enumerate(sizes)]
     fields[2] = synth.droplet(130, 40, 12.0, 0.9, densities=(0.42574, 1.65727))
     a, la = _run(P, descs, fields, (40,))
-    b, lb = _run(P, descs, fields, (40,), graph_steps=-1)
+    b, lb = _run(P, descs, fields, (40,), kernel_variant=P.LBM_KERNEL_TMA)
     assert (la, lb) == (1, 40)
     _same(a, b)
 
@@ -100,7 +101,8 @@ def test_handles_on_many_streams_at_once(P):
     for h in hs:
         P.lbm_destroy(h)
     for k, (nx, ny) in enumerate(sizes):
-        want, _ = _run(P, [_desc(P, nx, ny, 1, 0)], [_field(nx, ny, k)], (153,), graph_steps=-1)
+        want, _ = _run(P, [_desc(P, nx, ny, 1, 0)], [_field(nx, ny, k)], (153,),
+                       kernel_variant=P.LBM_KERNEL_TMA)
         _same([got[k]], want)
 
 
@@ -110,38 +112,44 @@ def test_handles_on_many_streams_at_once(P):
 ROW_SHAPES = [(901, 1403), (1200, 1100), (3, 40011), (61, 21001), (16001, 85), (2500, 1931)]
 
 
-@pytest.mark.parametrize("storage,mrt", [(1, 0), (1, 1), (2, 0), (2, 1)])
-def test_row_kernel_equals_tile_kernel(P, storage, mrt):
+@pytest.mark.parametrize("storage,mrt", [(1, 0), (0, 1), (2, 0), (2, 1)])
+def test_row_kernels_equal_tile_kernel(P, storage, mrt):
     for nx, ny in ROW_SHAPES:
         d, f = _desc(P, nx, ny, storage, mrt, sigma=0.5), _field(nx, ny)
-        a, la = _run(P, [d], [f], (5,))
-        b, lb = _run(P, [d], [f], (5,), kernel_variant=P.LBM_KERNEL_TMA)
-        assert la == lb == 5, (nx, ny)  # one launch a step: not resident
-        _same(a, b)
+        for kw in ({}, {"graph_steps": 2}, {"graph_steps": -1}):
+            # not resident: FP32 two steps a launch and the odd ones single
+            a, la = _run(P, [d], [f], (5, 1, 4), **kw)
+            assert la == (10 if storage == 2 else 6), (nx, ny)
+            b, lb = _run(P, [d], [f], (10,), kernel_variant=P.LBM_KERNEL_TMA) if not kw else (b, 10)
+            assert lb == 10
+            _same(a, b)
 
 
 @pytest.mark.parametrize("storage", [1, 2])
 def test_row_kernel_batches(P, storage):
-    sizes = [(700, 651), (3, 5), (61, 300), (800, 701), (33, 7), (640, 640)]
-    descs = [_desc(P, nx, ny, storage, 0, T=0.7 + 0.04 * k) for k, (nx, ny) in enumerate(sizes)]
+    sizes = [(700, 651), (3, 5), (61, 300), (2, 2), (800, 701), (33, 7), (640, 640), (57, 1)]
+    sizes = [(nx, max(ny, 2)) for nx, ny in sizes]
+    descs = [_desc(P, nx, ny, storage, 0, T=0.7 + 0.02 * k) for k, (nx, ny) in enumerate(sizes)]
     fields = [_field(nx, ny, k) for k, (nx, ny) in enumerate(sizes)]
-    a, la = _run(P, descs, fields, (5,))
-    b, lb = _run(P, descs, fields, (5,), kernel_variant=P.LBM_KERNEL_TMA)
-    assert la == lb == 5
+    a, la = _run(P, descs, fields, (35,))
+    b, lb = _run(P, descs, fields, (35,), kernel_variant=P.LBM_KERNEL_TMA)
+    assert (la, lb) == (35 if storage == 2 else 18, 35)
     _same(a, b)
 
 
-def test_served_fp16_results_equal_a_plain_handle(P):
-    # the server's FP16 requests run on row items, with step quotas
+@pytest.mark.parametrize("storage", [1, 2])
+def test_served_results_equal_a_plain_handle(P, storage):
+    # the server's requests run on row items with step quotas: two steps a
+    # launch in FP32 storage, odd quotas ending among even ones
     import time
 
     srv = P.lbm_server_create(P.lbm_server_opts_default(
         arena_bytes=1 << 30, max_request_sites=512 * 512, max_width=512, chunk_steps=7,
-        storage=P.LBM_STORE_F16_DEV))
-    reqs = [(100, 37, 20), (512, 300, 31), (61, 130, 5), (2, 3, 9), (400, 512, 13)]
+        storage=storage))
+    reqs = [(100, 37, 20), (512, 300, 31), (61, 130, 5), (2, 3, 1), (400, 512, 13), (57, 9, 2)]
     todo = {}
     for k, (nx, ny, n) in enumerate(reqs):
-        d, f = _desc(P, nx, ny, P.LBM_STORE_F16_DEV, 0), _field(nx, ny, k)
+        d, f = _desc(P, nx, ny, storage, 0), _field(nx, ny, k)
         todo[P.lbm_submit(srv, d, f, n)] = (d, f, n)
     while todo:
         for t in list(todo):
