@@ -259,13 +259,13 @@ __global__ void __launch_bounds__(512) k_fused(StepArgs a) {
 // (lbm_device.cuh, rest_finish): R(y) = f*_0(y) - w_0 rho0 rounded to the
 // storage type, G_i(y) = (f*_i(y) - w_i rho0) - c'_i (f*_0(y) - w_0 rho0)
 // + E/8 with E = 9/4 (exact R - stored R) = -9/4 e0.  Each thread writes
-// its own site, gathering the densities of its eight neighbours.  With
-// u = 0 (no velocity given) f^eq_i = w_i rho and
-// G_i(y) = w_i (rho(y + c_i) - rho(y)) - 9/32 e0: a subtraction and an FMA
-// per direction on the FP64 pipe (the slow one on GB300).
+// its own site.  With u = 0 (no velocity given: k_init) f^eq_i = w_i rho and
+// G_i(y) = w_i (rho(y + c_i) - rho(y)) - 9/32 e0, a subtraction and an FMA per
+// direction on the FP32 copy of the field (the differences of the rounded
+// values sum to zero over the lattice, so the stored mass stays that of the
+// FP64 field).
 template <class S>
-__global__ void k_init(LatDev L, void* pop, int parity, const double* rho, const float* rho32,
-                       const double* ux, const double* uy) {
+__global__ void k_init(LatDev L, void* pop, int parity, const double* rho, const float* rho32) {
     using T = typename S::T;
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
@@ -274,36 +274,75 @@ __global__ void k_init(LatDev L, void* pop, int parity, const double* rho, const
     T* o = reinterpret_cast<T*>(pop) + L.off_f[parity];
     const double w[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9,
                          1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
-    const bool still = !ux && !uy;
-    const double r0 = (double)L.rho0;
-    // f^eq_i - w_i rho0 at site (sx, sy), Eq. (SEDF)
-    auto geq = [&](int i, int sx, int sy) {
-        const int64_t q = (int64_t)sy * nx + sx;
-        const double r = rho[q];
-        if (still) return w[i] * (r - r0);
-        const double vx = ux ? ux[q] : 0.0, vy = uy ? uy[q] : 0.0;
-        const double cu = kCx[i] * vx + kCy[i] * vy;
-        return w[i] * (r + r * (3.0 * cu + 4.5 * cu * cu - 1.5 * (vx * vx + vy * vy))) - w[i] * r0;
-    };
-    const double g0 = geq(0, x, y);
+    const double g0 = w[0] * (rho[(int64_t)y * nx + x] - (double)L.rho0);
     const T R = S::cv((float)g0);
-    const double e0 = (double)S::rt((float)g0) - g0;
+    const float e0 = (float)((double)S::rt((float)g0) - g0);
     store_img(o, L.pitch, L.gx, x, y, nx, ny, R);
-    const float rc = rho32 ? rho32[(int64_t)y * nx + x] : 0.f;
-    const float e0f = (float)e0;
+    const float rc = rho32[(int64_t)y * nx + x];
 #pragma unroll
     for (int i = 1; i < 9; ++i) {
         int sx = x + kCx[i], sy = y + kCy[i];
         sx = sx < 0 ? sx + nx : (sx >= nx ? sx - nx : sx);
         sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
-        // u = 0: w_i (rho(y + c_i) - rho(y)) from the FP32 copy of the field
-        // (the differences of the rounded values sum to zero over the lattice,
-        // so the stored mass stays that of the FP64 field), e0 in FP32
-        const float G =
-            still && rho32
-                ? fmaf(-0.28125f, e0f, (float)w[i] * (rho32[(int64_t)sy * nx + sx] - rc))
-                : (float)((geq(i, sx, sy) - (double)cref(i) * g0) - 0.28125 * e0);
+        const float G = fmaf(-0.28125f, e0, (float)w[i] * (rho32[(int64_t)sy * nx + sx] - rc));
         store_img(o + i * L.plane, L.pitch, L.gx, x, y, nx, ny, S::cv(G));
+    }
+}
+
+// The same with a velocity.  Every site's nine FP64 equilibria are wanted by
+// nine threads (its own and its neighbours'), so a block computes those of
+// its 32 x 16 sites and one around them once, into shared memory: 612 x 47
+// FP64 operations for 512 sites instead of 512 x 99 (GB300 issues two a clock
+// and SM, which bounds this kernel): 4096^2 3.9 -> 3.0 ms.
+constexpr int kInitX = 32, kInitY = 16;
+constexpr size_t kInitSmem = sizeof(double) * 9 * (kInitX + 2) * (kInitY + 2);
+
+template <class S>
+__global__ void __launch_bounds__(256) k_init_u(LatDev L, void* pop, int parity, const double* rho,
+                                                const double* ux, const double* uy) {
+    using T = typename S::T;
+    constexpr int W = kInitX + 2, N = W * (kInitY + 2);
+    extern __shared__ double geq[];  // [9][kInitY + 2][kInitX + 2]
+    const int nx = L.nx, ny = L.ny;
+    const int x0 = blockIdx.x * kInitX, y0 = blockIdx.y * kInitY;
+    const double w[9] = {4.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9, 1.0 / 9,
+                         1.0 / 36, 1.0 / 36, 1.0 / 36, 1.0 / 36};
+    const double r0 = (double)L.rho0;
+    for (int k = threadIdx.x; k < N; k += blockDim.x) {
+        const int ly = k / W, lx = k - ly * W;
+        int sx = x0 + lx - 1, sy = y0 + ly - 1;
+        if (sx > nx || sy > ny) continue;  // beyond the last site's neighbours
+        sx = sx < 0 ? sx + nx : (sx >= nx ? sx - nx : sx);
+        sy = sy < 0 ? sy + ny : (sy >= ny ? sy - ny : sy);
+        const int64_t q = (int64_t)sy * nx + sx;
+        const double r = rho[q];
+        const double vx = ux ? ux[q] : 0.0, vy = uy ? uy[q] : 0.0;
+        // f^eq_i - w_i rho0, Eq. (SEDF)
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const int cx = plane_cx(i), cy = plane_cy(i);
+            const double ax = cx < 0 ? -vx : vx, ay = cy < 0 ? -vy : vy;
+            const double cu = cx ? (cy ? ax + ay : ax) : (cy ? ay : 0.0);
+            geq[i * N + k] = w[i] * (r + r * (3.0 * cu + 4.5 * cu * cu - 1.5 * (vx * vx + vy * vy))) -
+                             w[i] * r0;
+        }
+    }
+    __syncthreads();
+    T* o = reinterpret_cast<T*>(pop) + L.off_f[parity];
+    for (int k = threadIdx.x; k < kInitX * kInitY; k += blockDim.x) {
+        const int x = x0 + k % kInitX, y = y0 + k / kInitX;
+        if (x >= nx || y >= ny) continue;
+        const double* g = geq + (k / kInitX + 1) * W + k % kInitX + 1;
+        const double g0 = g[0];
+        const T R = S::cv((float)g0);
+        const double e0 = (double)S::rt((float)g0) - g0;
+        store_img(o, L.pitch, L.gx, x, y, nx, ny, R);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) {
+            const float G = (float)((g[i * N + plane_cy(i) * W + plane_cx(i)] - (double)cref(i) * g0) -
+                                    0.28125 * e0);
+            store_img(o + i * L.plane, L.pitch, L.gx, x, y, nx, ny, S::cv(G));
+        }
     }
 }
 
@@ -737,10 +776,17 @@ cudaError_t launch_init(int storage_f16, const LatDev& L, void* pop, int parity,
                         const double* rho, const float* rho32, const double* ux, const double* uy,
                         cudaStream_t st) {
     dim3 b(32, 8), g((L.nx + 31) / 32, (L.ny + 7) / 8);
-    if (storage_f16)
-        k_init<StoreF16><<<g, b, 0, st>>>(L, pop, parity, rho, rho32, ux, uy);
-    else
-        k_init<StoreF32><<<g, b, 0, st>>>(L, pop, parity, rho, rho32, ux, uy);
+    if (ux || uy) {
+        const dim3 gu((L.nx + kInitX - 1) / kInitX, (L.ny + kInitY - 1) / kInitY);
+        if (storage_f16)
+            k_init_u<StoreF16><<<gu, 256, kInitSmem, st>>>(L, pop, parity, rho, ux, uy);
+        else
+            k_init_u<StoreF32><<<gu, 256, kInitSmem, st>>>(L, pop, parity, rho, ux, uy);
+    } else if (storage_f16) {
+        k_init<StoreF16><<<g, b, 0, st>>>(L, pop, parity, rho, rho32);
+    } else {
+        k_init<StoreF32><<<g, b, 0, st>>>(L, pop, parity, rho, rho32);
+    }
     return cudaGetLastError();
 }
 

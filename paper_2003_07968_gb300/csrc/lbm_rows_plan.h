@@ -81,8 +81,8 @@ inline int pair_item_height(const std::vector<LatDev>& lats, int64_t pairs) {
     }
     return (int)std::min<int64_t>(h, most);
 }
-// 32-bit offsets: a lattice's rows in a plane take less than 4 GB
-inline bool pairs_fit(const LatDev& L, int es) {
+// 32-bit offsets of k_rows2: a lattice's rows in a plane take less than 4 GB
+inline bool rows_fit(const LatDev& L, int es) {
     return ((int64_t)L.ny + 2 * GY) * L.pitch * es < (int64_t)1 << 32;
 }
 

@@ -355,19 +355,18 @@ int make_resident(lbm_handle* h) {
     return LBM_OK;
 }
 
-// Row items of the handle's lattices, for k_rows and (where it can run) k_rows2.
+// Row items of the handle's lattices, for k_rows and then for k_rows2.  LBM_OK
+// without any where a lattice is too large for k_rows2.
 int make_items(lbm_handle* h) {
+    for (const LatDev& L : h->lat)
+        if (!rows_fit(L, h->f16 ? 2 : 4)) return LBM_OK;
     const int64_t sms = h->sm_count;
     std::vector<int4> t;
     const int height = row_item_height(h->lat, sms * 4 * kRowWarps);
     for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, height, t);
     const size_t n = t.size();
-    bool fit = true;
-    for (const LatDev& L : h->lat) fit = fit && pairs_fit(L, h->f16 ? 2 : 4);
-    if (fit) {
-        const int h2 = pair_item_height(h->lat, sms * 2 * kPairs);
-        for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, h2, t, kPairCols);
-    }
+    const int h2 = pair_item_height(h->lat, sms * 2 * kPairs);
+    for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, h2, t, kPairCols);
     h->items_bytes = t.size() * sizeof(int4);
     h->items = (int4*)dev_alloc(h, h->items_bytes);
     if (!h->items) return LBM_ERR_OOM;
@@ -1087,10 +1086,10 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
         const int rc = make_items(h);
         if (rc) return fail(rc);
-        h->path = tuned    ? tuned_path
-                  : h->f16 ? PATH_ROWS
-                           : PATH_PAIRS;  // measured: see k_rows2
-        if (h->path == PATH_PAIRS && !h->n_pair_items) h->path = PATH_ROWS;
+        h->path = !h->items ? PATH_TILES
+                  : tuned   ? tuned_path
+                  : h->f16  ? PATH_ROWS
+                            : PATH_PAIRS;  // measured: see k_rows2
     }
     h->tune_variant = variant;
     h->rec[0].name = "psi_pass";
@@ -1486,7 +1485,7 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
         if (k == 1 && h->items && rc == LBM_OK) {
             // the row kernels against the best tile kernel, per step
             h->path = PATH_TILES;
-            for (int two = 0; two < (h->n_pair_items ? 2 : 1); ++two) {
+            for (int two = 0; two < 2; ++two) {
                 cudaError_t e = launch_row_steps(h, h->parity, two);  // warm-up
                 cudaEventRecord(ea, h->stream);
                 for (int r = 0; r < repeats && e == cudaSuccess; ++r)

@@ -1053,13 +1053,13 @@ static int lbm_server_create_body(const lbm_server_opts* opts, lbm_server** out)
         S->pass[1].spt = kPassDefaults[1].spt;
     }
     // the row kernels, FP32 storage two steps a launch (where the tallest
-    // request's rows fit the 32-bit offsets of k_rows2)
-    S->rows = S->tma && o.kernel_variant == LBM_KERNEL_AUTO && o.eos_precision == LBM_EOS_DF &&
-              !(o.tile_x || o.tile_y);
+    // request's rows fit their 32-bit offsets)
     LatDev tallest{};
     tallest.pitch = (int32_t)S->pitch;
     tallest.ny = (int32_t)std::min<int64_t>(o.max_request_sites / 2, S->row_cap);
-    S->pairs = S->rows && !S->f16 && pairs_fit(tallest, S->es);
+    S->rows = S->tma && o.kernel_variant == LBM_KERNEL_AUTO && o.eos_precision == LBM_EOS_DF &&
+              !(o.tile_x || o.tile_y) && rows_fit(tallest, S->es);
+    S->pairs = S->rows && !S->f16;
     S->st.arena_bytes = (int64_t)o.arena_bytes;
     try {
         S->worker = std::thread(worker_main, S);
