@@ -3,8 +3,7 @@
 Default workload: one 8192 x 8192 FP32 droplet lattice (R = 2048, T_r = 0.8,
 BGK tau = 1, eps = 1.73, sigma = 1), the roofline configuration.  A "step"
 is one time step of the whole hot path over that lattice: pull, density,
-psi, force, collision and store, by default in one kernel launch (the
-single pass).  The working set (two population buffers, 4.8 GB) is far
+psi, force, collision and store, by default two steps in one kernel launch.  The working set (two population buffers, 4.8 GB) is far
 larger than L2, so no flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
@@ -431,12 +430,16 @@ def run_gpu(args):
                    "parallelism": f"replicas x{world}"},
         "roofline": {"bound": "hbm", "kernel": dom["name"], "achieved": round(achieved, 1),
                      "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
+                     # a launch of two steps moves the same bytes as one of one
+                     "steps_per_launch": 2 if dom["name"] == "fused_two_steps" else 1,
                      # the committed capture is of one kernel instance: the TMA single
                      # pass, 32x16 tiles, FP32 deviations, float-float EOS, BGK
                      "traffic": (ncu_traffic(dom["name"], wl["key"])
                                  if (args.collision, args.storage, args.eos, args.schedule,
-                                     info["collide_variant"], info["tile_x"], info["tile_y"])
-                                 == ("bgk", "f32dev", "df", "fused", P.LBM_KERNEL_TMA, 32, 16)
+                                     dom["name"], info["collide_variant"], info["tile_x"],
+                                     info["tile_y"])
+                                 == ("bgk", "f32dev", "df", "fused", "fused_step",
+                                     P.LBM_KERNEL_TMA, 32, 16)
                                  else None),
                      "peak_source": peak_src,
                      "bytes_per_launch": dom["bytes_per_launch"]},

@@ -93,7 +93,13 @@ extern "C" {
                               pass uses the TMA kernel with 32x16 tiles where
                               the population arena can be one tensor (one
                               lattice, or a batch in one row space), else
-                              plain loads with 32x8 tiles                    */
+                              plain loads with 32x8 tiles; with LBM_EOS_DF
+                              and no tile or grid given, kernels beside those
+                              take over: lattices that fit the SMs' shared
+                              memory advance many steps a launch, others in
+                              FP32 storage two, in FP16 storage one on a row
+                              kernel (lbm_info names the tile kernel, which
+                              takes the steps that are left)              */
 #define LBM_KERNEL_PLAIN 1 /* plain global loads, 1, 2 or 4 sites per thread
                               (with 2 or 4, site pairs share the paired FP32
                               instructions); tile_x a multiple of 32,
@@ -183,7 +189,9 @@ int lbm_init(lbm_handle* h, int32_t lattice, const double* rho, const double* ux
              const double* uy);
 
 /* Advance every lattice of the handle by nsteps >= 0 time steps.  Queues the
- * work and returns.  Reports an earlier numeric fault if one is already
+ * work and returns.  (Launches whose blocks wait for one another, those of
+ * many steps, are ordered on the device against such launches on other
+ * streams of the process where they would not fit the GPU together.)  Reports an earlier numeric fault if one is already
  * known.  Errors: LBM_ERR_ARG, LBM_ERR_CUDA, LBM_ERR_NUMERIC. */
 int lbm_step(lbm_handle* h, int64_t nsteps);
 
@@ -233,11 +241,13 @@ typedef struct {
 } lbm_kernel_stat;
 
 /* Waits, then reads the per-kernel records since lbm_profile(h, 1) into
- * out[0..max), returning the number of kernels in *n. */
+ * out[0..max), returning the number of kernels in *n: the psi pass, the
+ * single-pass (or collision) step and, where it ran, the launch of two
+ * steps.  While recording, no launch takes more than two steps. */
 int lbm_profile_read(lbm_handle* h, lbm_kernel_stat* out, int32_t max, int32_t* n);
 
 /* Number of kernels this handle has launched so far (graph replays count
- * each contained kernel). */
+ * each contained kernel; a launch of many steps counts once). */
 int64_t lbm_launch_count(lbm_handle* h);
 
 /* Handle facts: sites, device bytes held, and per pass (psi pass, collision
@@ -266,9 +276,9 @@ int lbm_autotune(lbm_handle* h, int32_t repeats);
 
 /* ---- serving: continuous batching --------------------------------------- */
 /* A server keeps many independent lattices (requests) resident in one
- * device arena and steps all of them together: every chunk of steps is one
- * pair of launches per step over a tile list that spans every resident
- * lattice (the same kernels as a batch handle).  Requests are admitted at
+ * device arena and steps all of them together: a chunk of steps is a launch
+ * per step, or per two steps in FP32 storage, over a list that spans every
+ * resident lattice (the same kernels as a batch handle).  Requests are admitted at
  * chunk boundaries, first come first served but skipping any that do not
  * fit yet, whenever a slot and arena space (HBM footprint: both population
  * buffers at the arena's common pitch, plus psi) are free and the resident

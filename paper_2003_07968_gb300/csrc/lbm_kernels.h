@@ -79,16 +79,16 @@ cudaError_t launch_fused_tma(int f16, int mrt, int eos, int tx, int ty, const St
                              cudaStream_t st);
 int occupancy_fused_tma(int f16, int mrt, int eos, int tx, int ty, bool with_map, bool single);
 // One step, a warp an item (a.tiles: row items, lbm_rows_plan.h; float-float
-// EOS); lat0 as in launch_fused_tma.
+// EOS); lat0 as in launch_fused_tma.  FP32 storage: BGK batches only.
 cudaError_t launch_rows(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st);
-// Two steps, a pair of warps an item (a.tiles: row items of kPairCols; float-
-// float EOS; lattices of less than 4 GB a plane).
+// Two steps, a pair of warps an item (a.tiles: row items of kPairCols; FP32
+// storage, float-float EOS, lattices for which rows_fit).
 cudaError_t launch_pairs(int f16, int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st);
 // Many steps in one cooperative launch over a resident plan's tiles
 // (float-float EOS; lbm_rows.cuh): lat0 as in launch_fused_tma.  All blocks
 // must be resident together: grid at most SMs x resident_blocks_per_sm.
 cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
                             size_t smem, cudaStream_t st);
-int resident_blocks_per_sm(int f16, int mrt, bool single, size_t smem);
+int resident_blocks_per_sm(int f16, int mrt, bool single);
 
 }  // namespace pplbm

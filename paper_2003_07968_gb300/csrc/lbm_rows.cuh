@@ -768,13 +768,10 @@ cudaError_t resident_inst(const ResArgs* m, const LatDev* lat0, int grid, size_t
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(32 * kResWarps), p, smem, st);
 }
 
-template <class S, bool MRT>
+template <class S, bool MRT, bool ONE>
 cudaError_t rows_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
     const unsigned grid = (unsigned)((a.ntiles + kRowWarps - 1) / kRowWarps);
-    if (lat0)
-        k_rows<S, EOS_DF, MRT, true><<<grid, 32 * kRowWarps, 0, st>>>(a, *lat0);
-    else
-        k_rows<S, EOS_DF, MRT, false><<<grid, 32 * kRowWarps, 0, st>>>(a, LatDev{});
+    k_rows<S, EOS_DF, MRT, ONE><<<grid, 32 * kRowWarps, 0, st>>>(a, lat0 ? *lat0 : LatDev{});
     return cudaGetLastError();
 }
 
@@ -791,15 +788,22 @@ cudaError_t pairs_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
 
 }  // namespace
 
+// (FP32 storage only, see k_rows2)
 template <class S>
 cudaError_t pairs_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
     if (mrt) return lat0 ? pairs_inst<S, true, true>(a, lat0, st) : pairs_inst<S, true, false>(a, lat0, st);
     return lat0 ? pairs_inst<S, false, true>(a, lat0, st) : pairs_inst<S, false, false>(a, lat0, st);
 }
 
+// (FP32 storage: the odd steps of a server's requests only)
 template <class S>
 cudaError_t rows_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
-    return mrt ? rows_inst<S, true>(a, lat0, st) : rows_inst<S, false>(a, lat0, st);
+    if constexpr (sizeof(typename S::T) == 4)
+        return mrt || lat0 ? cudaErrorInvalidValue : rows_inst<S, false, false>(a, nullptr, st);
+    else if (mrt)
+        return lat0 ? rows_inst<S, true, true>(a, lat0, st) : rows_inst<S, true, false>(a, nullptr, st);
+    else
+        return lat0 ? rows_inst<S, false, true>(a, lat0, st) : rows_inst<S, false, false>(a, nullptr, st);
 }
 
 // One storage type: the launch (occ null), or its blocks per SM into *occ

@@ -12,8 +12,4 @@ cudaError_t rows_f16(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_
     return rows_any<StoreF16>(mrt, a, lat0, st);
 }
 
-cudaError_t pairs_f16(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
-    return pairs_any<StoreF16>(mrt, a, lat0, st);
-}
-
 }  // namespace pplbm

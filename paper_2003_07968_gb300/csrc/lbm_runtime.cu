@@ -49,7 +49,7 @@ struct PassCfg {
     int variant, tx, ty, grid, spt;
 };
 // What the single pass runs on: the tile kernels of pass[1], k_rows, or
-// k_rows2 (two steps a launch, an odd step on k_rows).
+// k_rows2 (two steps a launch, an odd step on the tile kernel).
 enum StepPath { PATH_TILES, PATH_ROWS, PATH_PAIRS };
 struct TuneVal {
     PassCfg pass[2];
@@ -120,8 +120,8 @@ struct lbm_handle {
     cudaEvent_t chunk_ev[5] = {};
     int64_t device_bytes = 0;
     // host side
-    uint32_t* status_host = nullptr;  // pinned
-    double* scan_host = nullptr;      // pinned: lbm_init's field scan result
+    double* scan_host = nullptr;      // pinned: a device result (lbm_init's scan, the mass)
+    uint32_t* status_host = nullptr;  // ... and the fault words after it
     cudaEvent_t status_ev = nullptr;
     bool status_pending = false;
     int32_t starve = 0;        // armed failure-detection test (tile + 1), for one launch
@@ -142,9 +142,9 @@ struct lbm_handle {
     // wide); else that kernel uses row copies
     CUtensorMap tmap[2]{};  // loads, stores
     bool has_tmap = false;
-    // row items of the lattices for k_rows, then for k_rows2 (none: not built)
+    // row items of the lattices for the row kernel of their storage (none: no plan)
     int4* items = nullptr;
-    int n_items = 0, n_pair_items = 0;
+    int n_items = 0;
     size_t items_bytes = 0;
     StepPath path = PATH_TILES;
     // the lattices as resident tiles, when they fit (plan_resident): tiles,
@@ -340,8 +340,8 @@ int make_resident(lbm_handle* h) {
         return LBM_OK;
     const ResPlan P = plan_resident(h->lat, std::min(2 * h->sm_count, kResBlocks), h->f16 ? 2 : 4);
     if (P.tiles.empty()) return LBM_OK;
-    const int per_sm = resident_blocks_per_sm(h->f16, h->collision == LBM_COLL_MRT,
-                                              h->lat.size() == 1, P.smem);
+    const int per_sm =
+        resident_blocks_per_sm(h->f16, h->collision == LBM_COLL_MRT, h->lat.size() == 1);
     if (per_sm < 2) return LBM_OK;  // the flights are counted at two blocks an SM
     h->res_grid = (int)P.tiles.size();
     h->res_smem = P.smem;
@@ -355,34 +355,33 @@ int make_resident(lbm_handle* h) {
     return LBM_OK;
 }
 
-// Row items of the handle's lattices, for k_rows and then for k_rows2.  LBM_OK
-// without any where a lattice is too large for k_rows2.
+// Row items of the handle's lattices: for k_rows (FP16 storage) or k_rows2
+// (FP32).  LBM_OK without any where a lattice is too large for them.
 int make_items(lbm_handle* h) {
     for (const LatDev& L : h->lat)
         if (!rows_fit(L, h->f16 ? 2 : 4)) return LBM_OK;
     const int64_t sms = h->sm_count;
+    const int height = h->f16 ? row_item_height(h->lat, sms * 4 * kRowWarps)
+                              : pair_item_height(h->lat, sms * 2 * kPairs);
     std::vector<int4> t;
-    const int height = row_item_height(h->lat, sms * 4 * kRowWarps);
-    for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, height, t);
-    const size_t n = t.size();
-    const int h2 = pair_item_height(h->lat, sms * 2 * kPairs);
-    for (size_t l = 0; l < h->lat.size(); ++l) row_items(h->lat[l], (int)l, h2, t, kPairCols);
+    for (size_t l = 0; l < h->lat.size(); ++l)
+        row_items(h->lat[l], (int)l, height, t, h->f16 ? kRowCols : kPairCols);
     h->items_bytes = t.size() * sizeof(int4);
     h->items = (int4*)dev_alloc(h, h->items_bytes);
     if (!h->items) return LBM_ERR_OOM;
     CK(h, cudaMemcpyAsync(h->items, t.data(), h->items_bytes, cudaMemcpyHostToDevice, h->stream));
-    h->n_items = (int)n;
-    h->n_pair_items = (int)(t.size() - n);
+    h->n_items = (int)t.size();
     return LBM_OK;
 }
 
-// One step on k_rows, or two on k_rows2, from buffer `parity` to the other.
-cudaError_t launch_row_steps(lbm_handle* h, int parity, bool two) {
+// The row kernel over the handle's items, from buffer `parity` to the other:
+// one step (FP16 storage) or two (FP32).
+cudaError_t launch_row_steps(lbm_handle* h, int parity) {
     StepArgs a = step_args(h, parity, 1);
-    a.tiles = h->items + (two ? h->n_items : 0);
-    a.ntiles = two ? h->n_pair_items : h->n_items;
-    return (two ? launch_pairs : launch_rows)(h->f16, h->collision == LBM_COLL_MRT, a,
-                                              h->lat.size() == 1 ? &h->lat[0] : nullptr, h->stream);
+    a.tiles = h->items;
+    a.ntiles = h->n_items;
+    return (h->f16 ? launch_rows : launch_pairs)(h->f16, h->collision == LBM_COLL_MRT, a,
+                                                 h->lat.size() == 1 ? &h->lat[0] : nullptr, h->stream);
 }
 
 // nsteps steps in one launch (state from buffer `parity` to the other).
@@ -481,8 +480,8 @@ int launch_step(lbm_handle* h, int p) {
     a1.starve = h->starve;  // an armed failure-detection test goes into this launch only
     if (h->starve) a1.wait_cycles = kTestWaitBudgetCycles;
     h->starve = 0;
-    if (h->path != PATH_TILES && !a1.starve)
-        CK(h, launch_row_steps(h, p, false));
+    if (h->path == PATH_ROWS && !a1.starve)
+        CK(h, launch_row_steps(h, p));
     else
         CK(h, launch_pass(h, 1, a1, h->pass[1].grid));
     if (h->prof) {
@@ -503,7 +502,7 @@ int launch_two_steps(lbm_handle* h, int p) {
         e2 = take_event(h);
         CK(h, cudaEventRecord(e1, h->stream));
     }
-    CK(h, launch_row_steps(h, p, true));
+    CK(h, launch_row_steps(h, p));
     if (h->prof) {
         CK(h, cudaEventRecord(e2, h->stream));
         h->rec[2].pending.emplace_back(e1, e2);
@@ -628,7 +627,6 @@ void release(lbm_handle* h) {
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     h->ev_pool.clear();
     if (h->status_ev) cudaEventDestroy(h->status_ev);
-    if (h->status_host) cudaFreeHost(h->status_host);
     if (h->scan_host) cudaFreeHost(h->scan_host);
     dev_free(h, h->staging, staging_bytes(h->staging_elems));
     dev_free(h, h->partials, (kMassPartials + 1) * sizeof(double));
@@ -1020,9 +1018,12 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
     h->partials = (double*)dev_alloc(h, (kMassPartials + 1) * sizeof(double));
     if (!h->pop || !h->psi || !h->lat_dev || !h->status || !h->partials)
         return fail(LBM_ERR_OOM);
-    if (cudaMallocHost(&h->status_host, n * sizeof(uint32_t)) != cudaSuccess ||
-        cudaMallocHost(&h->scan_host, sizeof(double)) != cudaSuccess)
+    // one page-locked block (each allocation of its own costs about 0.1 ms)
+    if (cudaMallocHost(&h->scan_host, sizeof(double) + n * sizeof(uint32_t)) != cudaSuccess) {
+        h->scan_host = nullptr;
         return fail(LBM_ERR_OOM);
+    }
+    h->status_host = reinterpret_cast<uint32_t*>(h->scan_host + 1);
     if (cudaEventCreateWithFlags(&h->status_ev, cudaEventDisableTiming) != cudaSuccess ||
         cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking) != cudaSuccess)
         return fail(LBM_ERR_CUDA);
@@ -1167,13 +1168,16 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     int rc = check_status_async(h);
     if (rc) return rc;
     int64_t left = nsteps;
+    // Into a caller's stream capture goes one launch per step: a replayed graph
+    // would not be counted among the resident launches in flight, and must end
+    // in the buffer that an even number of steps ends in.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (h->res_grid || h->path == PATH_PAIRS) CK(h, cudaStreamIsCapturing(h->stream, &cap));
+    const bool many = cap == cudaStreamCaptureStatusNone;
     // resident lattices: from two steps on (one step is one tile-kernel launch;
-    // a resident one costs about 3 us beside its steps).  Not into a caller's
-    // stream capture: a replayed graph would not be counted among the flights.
+    // a resident one costs about 3 us beside its steps)
     if (h->res_grid && left >= 2 && !h->prof && !h->starve) {
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        CK(h, cudaStreamIsCapturing(h->stream, &cap));
-        while (cap == cudaStreamCaptureStatusNone && left >= 2) {
+        while (many && left >= 2) {
             // at most 2^14 steps a launch (a fraction of a second)
             const int n = (int)std::min<int64_t>(left, left == (1 << 14) + 1 ? 1 << 13 : 1 << 14);
             rc = launch_resident_steps(h, n);
@@ -1194,7 +1198,7 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
         if (h->path == PATH_PAIRS && (h->graph_launches & 1)) h->parity ^= 1;
     }
     while (left > 0) {
-        const bool two = h->path == PATH_PAIRS && left >= 2 && !h->starve;
+        const bool two = h->path == PATH_PAIRS && many && left >= 2 && !h->starve;
         rc = two ? launch_two_steps(h, h->parity) : launch_step(h, h->parity);
         if (rc) return rc;
         h->parity ^= 1;
@@ -1483,24 +1487,18 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
         h->pass[k].grid = bc.grid;
         best_cfg.pass[k] = bc;
         if (k == 1 && h->items && rc == LBM_OK) {
-            // the row kernels against the best tile kernel, per step
+            // the row kernel against the best tile kernel, per step
+            const StepPath row = h->f16 ? PATH_ROWS : PATH_PAIRS;
             h->path = PATH_TILES;
-            for (int two = 0; two < 2; ++two) {
-                cudaError_t e = launch_row_steps(h, h->parity, two);  // warm-up
-                cudaEventRecord(ea, h->stream);
-                for (int r = 0; r < repeats && e == cudaSuccess; ++r)
-                    e = launch_row_steps(h, h->parity, two);
-                cudaEventRecord(eb, h->stream);
-                if (e == cudaSuccess) e = cudaEventSynchronize(eb);
-                if (e != cudaSuccess) { rc = cuda_fail(h, e, "autotune rows"); break; }
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, ea, eb);
-                if (two) ms *= 0.5f;
-                if (ms < best) {
-                    best = ms;
-                    h->path = two ? PATH_PAIRS : PATH_ROWS;
-                }
-            }
+            cudaError_t e = launch_row_steps(h, h->parity);  // warm-up
+            cudaEventRecord(ea, h->stream);
+            for (int r = 0; r < repeats && e == cudaSuccess; ++r) e = launch_row_steps(h, h->parity);
+            cudaEventRecord(eb, h->stream);
+            if (e == cudaSuccess) e = cudaEventSynchronize(eb);
+            if (e != cudaSuccess) { rc = cuda_fail(h, e, "autotune rows"); break; }
+            float ms = 0.f;
+            cudaEventElapsedTime(&ms, ea, eb);
+            if (ms < best * (row == PATH_PAIRS ? 2.f : 1.f)) h->path = row;
             best_cfg.path = h->path;
         }
     }

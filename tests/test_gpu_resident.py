@@ -186,3 +186,26 @@ def test_fields_read_back_into_any_host_array(P):
             got = P.lbm_moments(h, 0, out=dict(zip(("rho", "ux", "uy"), mix)))
             _same([got], [want])
         P.lbm_destroy(h)
+
+
+def test_steps_captured_by_the_caller_replay(P):
+    # into a caller's capture goes one launch per step, so that a replay of an
+    # even number of steps ends in the buffer it started from
+    import torch
+
+    for nx, ny in ((64, 50), (1100, 901)):
+        d, f = _desc(P, nx, ny, 1, 0), _field(nx, ny)
+        h = P.lbm_create(d)
+        P.lbm_init(h, 0, f)
+        P.lbm_step(h, 4)
+        P.lbm_sync(h)
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=h.stream):
+            P.lbm_step(h, 2)
+        with torch.cuda.stream(h.stream):
+            for _ in range(3):
+                g.replay()
+        got = P.lbm_moments(h, 0)
+        P.lbm_destroy(h)
+        want, _ = _run(P, [d], [f], (10,), kernel_variant=P.LBM_KERNEL_TMA)
+        _same([got], want)
