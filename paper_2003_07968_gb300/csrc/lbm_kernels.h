@@ -88,7 +88,7 @@ cudaError_t launch_pairs(int f16, int mrt, const StepArgs& a, const LatDev* lat0
 // (float-float EOS; lbm_rows.cuh): lat0 as in launch_fused_tma.  All blocks
 // must be resident together: grid at most SMs x resident_blocks_per_sm.
 cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
-                            size_t smem, cudaStream_t st);
+                            cudaStream_t st);
 int resident_blocks_per_sm(int f16, int mrt, bool single);
 
 }  // namespace pplbm

@@ -8,8 +8,8 @@
 
 namespace pplbm {
 
-cudaError_t resident_f32(int, const ResArgs*, const LatDev*, int, size_t, cudaStream_t, int*);
-cudaError_t resident_f16(int, const ResArgs*, const LatDev*, int, size_t, cudaStream_t, int*);
+cudaError_t resident_f32(int, const ResArgs*, const LatDev*, int, cudaStream_t, int*);
+cudaError_t resident_f16(int, const ResArgs*, const LatDev*, int, cudaStream_t, int*);
 
 cudaError_t rows_f32(int, const StepArgs&, const LatDev*, cudaStream_t);
 cudaError_t rows_f16(int, const StepArgs&, const LatDev*, cudaStream_t);
@@ -25,8 +25,8 @@ cudaError_t launch_pairs(int f16, int mrt, const StepArgs& a, const LatDev* lat0
 }
 
 cudaError_t launch_resident(int f16, int mrt, const ResArgs& m, const LatDev* lat0, int grid,
-                            size_t smem, cudaStream_t st) {
-    return (f16 ? resident_f16 : resident_f32)(mrt, &m, lat0, grid, smem, st, nullptr);
+                            cudaStream_t st) {
+    return (f16 ? resident_f16 : resident_f32)(mrt, &m, lat0, grid, st, nullptr);
 }
 
 int resident_blocks_per_sm(int f16, int mrt, bool single) {
@@ -42,7 +42,7 @@ int resident_blocks_per_sm(int f16, int mrt, bool single) {
     int occ = 0;
     const LatDev lat{};
     const cudaError_t e = (f16 ? resident_f16 : resident_f32)(mrt, nullptr, single ? &lat : nullptr,
-                                                             0, kResSmem, nullptr, &occ);
+                                                             0, nullptr, &occ);
     if (e != cudaSuccess) return 0;
     known[key] = occ;
     return occ;

@@ -756,16 +756,15 @@ __global__ void __launch_bounds__(32 * kResWarps, 2)
 
 // ---------------------------------------------------------------- launchers
 template <class S, bool MRT, bool ONE>
-cudaError_t resident_inst(const ResArgs* m, const LatDev* lat0, int grid, size_t smem,
-                          cudaStream_t st, int* occ) {
+cudaError_t resident_inst(const ResArgs* m, const LatDev* lat0, int grid, cudaStream_t st, int* occ) {
     const void* fn = (const void*)k_resident<S, EOS_DF, MRT, ONE>;
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kResSmem);
     if (e != cudaSuccess) return e;
-    if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, fn, 32 * kResWarps, smem);
+    if (occ) return cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, fn, 32 * kResWarps, kResSmem);
     ResArgs args = *m;
     LatDev lat = lat0 ? *lat0 : LatDev{};
     void* p[] = {&args, &lat};
-    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(32 * kResWarps), p, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(32 * kResWarps), p, kResSmem, st);
 }
 
 template <class S, bool MRT, bool ONE>
@@ -809,13 +808,13 @@ cudaError_t rows_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_
 // One storage type: the launch (occ null), or its blocks per SM into *occ
 // (lat0 not null: one lattice).
 template <class S>
-cudaError_t resident_any(int mrt, const ResArgs* m, const LatDev* lat0, int grid, size_t smem,
-                         cudaStream_t st, int* occ) {
+cudaError_t resident_any(int mrt, const ResArgs* m, const LatDev* lat0, int grid, cudaStream_t st,
+                         int* occ) {
     if (mrt)
-        return lat0 ? resident_inst<S, true, true>(m, lat0, grid, smem, st, occ)
-                    : resident_inst<S, true, false>(m, lat0, grid, smem, st, occ);
-    return lat0 ? resident_inst<S, false, true>(m, lat0, grid, smem, st, occ)
-                : resident_inst<S, false, false>(m, lat0, grid, smem, st, occ);
+        return lat0 ? resident_inst<S, true, true>(m, lat0, grid, st, occ)
+                    : resident_inst<S, true, false>(m, lat0, grid, st, occ);
+    return lat0 ? resident_inst<S, false, true>(m, lat0, grid, st, occ)
+                : resident_inst<S, false, false>(m, lat0, grid, st, occ);
 }
 
 }  // namespace pplbm

@@ -3,9 +3,9 @@
 
 namespace pplbm {
 
-cudaError_t resident_f32(int mrt, const ResArgs* m, const LatDev* lat0, int grid, size_t smem,
+cudaError_t resident_f32(int mrt, const ResArgs* m, const LatDev* lat0, int grid,
                          cudaStream_t st, int* occ) {
-    return resident_any<StoreF32>(mrt, m, lat0, grid, smem, st, occ);
+    return resident_any<StoreF32>(mrt, m, lat0, grid, st, occ);
 }
 
 cudaError_t rows_f32(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {

@@ -88,7 +88,9 @@ inline bool rows_fit(const LatDev& L, int es) {
 
 // ---- resident lattices: one tile a block, kept in shared memory for many steps
 constexpr int kResWarps = 8;            // warps of a block, one row each at a time
-constexpr int kResSmem = 113 * 1024;    // shared memory of a block (two on an SM)
+// shared memory of a block: half an SM's, whatever its tile needs, so that any
+// two blocks of any launches share an SM (launches in flight are counted so)
+constexpr int kResSmem = 113 * 1024;
 constexpr int kResRows = 96;            // rows of a tile at most
 constexpr int kResMail = 1088;          // packets of a mailbox slot at most
 constexpr int kResBlocks = 480;         // blocks of a launch at most
@@ -132,7 +134,6 @@ inline int res_bands(int ny, int rows) { return std::max(1, std::min((ny + rows 
 
 struct ResPlan {
     std::vector<ResTile> tiles;  // none: no plan
-    size_t smem = 0;
     int rows = 0;  // of the tallest tile
 };
 
@@ -155,7 +156,6 @@ inline ResPlan plan_resident(const std::vector<LatDev>& lats, int blocks, int es
         }
         if (n <= blocks && tallest <= most) {
             h = rows;
-            P.smem = res_smem(tallest, kRowCols, es);
             P.rows = tallest;
         }
     }

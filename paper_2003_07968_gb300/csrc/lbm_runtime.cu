@@ -150,7 +150,7 @@ struct lbm_handle {
     // the lattices as resident tiles, when they fit (plan_resident): tiles,
     // mailboxes and epochs in one allocation
     int res_grid = 0;  // tiles (0: no plan)
-    size_t res_smem = 0, res_bytes = 0;
+    size_t res_bytes = 0;
     int res_slot = 0;
     void* res = nullptr;
     bool res_reset = true;  // mailboxes and epochs must be cleared first
@@ -344,7 +344,6 @@ int make_resident(lbm_handle* h) {
         resident_blocks_per_sm(h->f16, h->collision == LBM_COLL_MRT, h->lat.size() == 1);
     if (per_sm < 2) return LBM_OK;  // the flights are counted at two blocks an SM
     h->res_grid = (int)P.tiles.size();
-    h->res_smem = P.smem;
     h->res_slot = res_packets(P.rows, kRowCols);
     h->res_bytes = res_epoch_off(h) + h->res_grid * sizeof(uint32_t);
     h->res = dev_alloc(h, h->res_bytes);
@@ -434,7 +433,7 @@ int launch_resident_steps(lbm_handle* h, int nsteps) {
     }
     const cudaError_t e =
         launch_resident(h->f16, h->collision == LBM_COLL_MRT, m,
-                        h->lat.size() == 1 ? &h->lat[0] : nullptr, h->res_grid, h->res_smem, h->stream);
+                        h->lat.size() == 1 ? &h->lat[0] : nullptr, h->res_grid, h->stream);
     if (e == cudaSuccess) mine->blocks = std::max(mine->blocks, h->res_grid);
     // (a record after a failed launch only marks the work queued before it)
     const cudaError_t r = cudaEventRecord(mine->done, h->stream);
