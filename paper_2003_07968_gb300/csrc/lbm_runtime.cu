@@ -237,6 +237,7 @@ int build_tiles(lbm_handle* h, int k, int tx, int ty) {
     }
     const size_t bytes = t.size() * sizeof(int4);
     if (bytes > P.cap) {
+        if (P.tiles) CK(h, cudaStreamSynchronize(h->stream));  // no launch reads the old list
         dev_free(h, P.tiles, P.cap);
         P.tiles = (int4*)dev_alloc(h, bytes);
         if (!P.tiles) {
@@ -245,8 +246,8 @@ int build_tiles(lbm_handle* h, int k, int tx, int ty) {
         }
         P.cap = bytes;
     }
+    // (a copy from pageable memory has read it when the call returns)
     CK(h, cudaMemcpyAsync(P.tiles, t.data(), bytes, cudaMemcpyHostToDevice, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     P.tx = tx;
     P.ty = ty;
     P.ntiles = (int)t.size();
