@@ -191,8 +191,10 @@ int lbm_init(lbm_handle* h, int32_t lattice, const double* rho, const double* ux
 /* Advance every lattice of the handle by nsteps >= 0 time steps.  Queues the
  * work and returns.  (Launches whose blocks wait for one another, those of
  * many steps, are ordered on the device against such launches on other
- * streams of the process where they would not fit the GPU together.)  Reports an earlier numeric fault if one is already
- * known.  Errors: LBM_ERR_ARG, LBM_ERR_CUDA, LBM_ERR_NUMERIC. */
+ * streams of the process where they would not fit the GPU together.)  While
+ * the handle's stream is being captured by the caller, one launch per step is
+ * recorded, whatever nsteps is.  Reports an earlier numeric fault if one is
+ * already known.  Errors: LBM_ERR_ARG, LBM_ERR_CUDA, LBM_ERR_NUMERIC. */
 int lbm_step(lbm_handle* h, int64_t nsteps);
 
 /* Macroscopic fields of one lattice at the current time: rho (Eq. FD), the

@@ -1165,19 +1165,20 @@ int lbm_init(lbm_handle* h, int32_t lattice, const double* rho, const double* ux
 
 static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     if (!h || nsteps < 0) return LBM_ERR_ARG;
-    int rc = check_status_async(h);
+    // Into a caller's stream capture goes one launch per step and nothing else:
+    // a graph of the handle's own can be neither captured nor launched there, a
+    // replayed resident launch would not be counted among those in flight, an
+    // event queried ends the capture, and one recorded there cannot be queried.
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CK(h, cudaStreamIsCapturing(h->stream, &cap));
+    const bool direct = cap == cudaStreamCaptureStatusNone;
+    int rc = direct ? check_status_async(h) : fault_code(h);
     if (rc) return rc;
     int64_t left = nsteps;
-    // Into a caller's stream capture goes one launch per step: a replayed graph
-    // would not be counted among the resident launches in flight, and must end
-    // in the buffer that an even number of steps ends in.
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (h->res_grid || h->path == PATH_PAIRS) CK(h, cudaStreamIsCapturing(h->stream, &cap));
-    const bool many = cap == cudaStreamCaptureStatusNone;
     // resident lattices: from two steps on (one step is one tile-kernel launch;
     // a resident one costs about 3 us beside its steps)
-    if (h->res_grid && left >= 2 && !h->prof && !h->starve) {
-        while (many && left >= 2) {
+    if (direct && h->res_grid && left >= 2 && !h->prof && !h->starve) {
+        while (left >= 2) {
             // at most 2^14 steps a launch (a fraction of a second)
             const int n = (int)std::min<int64_t>(left, left == (1 << 14) + 1 ? 1 << 13 : 1 << 14);
             rc = launch_resident_steps(h, n);
@@ -1186,7 +1187,7 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
             left -= n;
         }
     }
-    while (!h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps) {
+    while (direct && !h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps) {
         if (!h->graph[h->parity]) {
             rc = capture_graph(h);
             if (rc) return rc;
@@ -1198,13 +1199,13 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
         if (h->path == PATH_PAIRS && (h->graph_launches & 1)) h->parity ^= 1;
     }
     while (left > 0) {
-        const bool two = h->path == PATH_PAIRS && many && left >= 2 && !h->starve;
+        const bool two = h->path == PATH_PAIRS && direct && left >= 2 && !h->starve;
         rc = two ? launch_two_steps(h, h->parity) : launch_step(h, h->parity);
         if (rc) return rc;
         h->parity ^= 1;
         left -= two ? 2 : 1;
     }
-    if (!h->status_pending) {
+    if (direct && !h->status_pending) {
         CK(h, cudaMemcpyAsync(h->status_host, h->status, h->lat.size() * sizeof(uint32_t),
                               cudaMemcpyDeviceToHost, h->stream));
         CK(h, cudaEventRecord(h->status_ev, h->stream));

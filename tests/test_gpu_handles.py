@@ -1,0 +1,89 @@
+"""What a handle keeps between calls: the buffer its state is in, the graphs
+that callers capture around lbm_step, tuned choices and records.
+
+Every kernel runs the same operations on the same values, so a handle's
+fields are compared bit for bit with those of one that takes every step on
+the tile kernel (kernel_variant=LBM_KERNEL_TMA).
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def P():
+    import torch
+
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2003_07968_gb300 import build, capi
+
+    build.build()
+    capi.load()
+    return capi
+
+
+def _field(nx, ny, k=0):
+    rng = np.random.default_rng(17 + k)
+    rho = synth.droplet(nx, ny, 0.3 * min(nx, ny) + 1, 0.8)
+    return rho + 1e-3 * rng.standard_normal(rho.shape)
+
+
+def _tile_run(P, desc, field, nsteps):
+    h = P.lbm_create(desc, kernel_variant=P.LBM_KERNEL_TMA)
+    P.lbm_init(h, 0, field)
+    P.lbm_step(h, nsteps)
+    out = P.lbm_moments(h, 0)
+    P.lbm_destroy(h)
+    return out
+
+
+def _same(x, y):
+    for k in ("rho", "ux", "uy"):
+        assert np.array_equal(x[k], y[k]), k
+    assert x["mass"] == y["mass"]
+
+
+def _capture(P, h, nsteps):
+    import torch
+
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=h.stream):
+        P.lbm_step(h, nsteps)
+    return g
+
+
+def _replay(h, g):
+    import torch
+
+    with torch.cuda.stream(h.stream):
+        g.replay()
+
+
+# ------------------------------------------------ graphs captured by the caller
+# (sites, storage): resident, two steps a launch, one step a launch on rows
+KINDS = [((64, 50), 1), ((1100, 901), 1), ((1100, 901), 2)]
+
+
+@pytest.mark.parametrize("shape,storage", KINDS)
+@pytest.mark.parametrize("kw", [{}, {"graph_steps": 2}])
+def test_captured_steps_are_single_launches(P, shape, storage, kw):
+    # a captured call of graph_steps steps or more, on a handle that has
+    # graphs of its own (or none: resident): an even number of steps can be
+    # replayed any number of times
+    d, f = P.lbm_desc_default(*shape, T=0.8, storage=storage), _field(*shape)
+    for warm in (4, 34, 33):
+        h = P.lbm_create(d, **kw)
+        P.lbm_init(h, 0, f)
+        P.lbm_step(h, warm)
+        l0 = P.lbm_launch_count(h)
+        g = _capture(P, h, 34)
+        assert P.lbm_launch_count(h) - l0 == 34
+        for _ in range(3):
+            _replay(h, g)
+        P.lbm_step(h, 1)  # the capture left no event behind that this one queries
+        got = P.lbm_moments(h, 0)
+        P.lbm_destroy(h)
+        _same(got, _tile_run(P, d, f, warm + 3 * 34 + 1))
