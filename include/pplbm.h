@@ -193,7 +193,10 @@ int lbm_init(lbm_handle* h, int32_t lattice, const double* rho, const double* ux
  * many steps, are ordered on the device against such launches on other
  * streams of the process where they would not fit the GPU together.)  While
  * the handle's stream is being captured by the caller, one launch per step is
- * recorded, whatever nsteps is.  Reports an earlier numeric fault if one is
+ * recorded, whatever nsteps is; a graph captured over an even number of steps
+ * may be replayed after any even number of further steps (replays or calls of
+ * this function), until lbm_init or lbm_autotune changes what its launches
+ * carry.  Reports an earlier numeric fault if one is
  * already known.  Errors: LBM_ERR_ARG, LBM_ERR_CUDA, LBM_ERR_NUMERIC. */
 int lbm_step(lbm_handle* h, int64_t nsteps);
 

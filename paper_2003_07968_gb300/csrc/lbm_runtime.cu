@@ -136,6 +136,11 @@ struct lbm_handle {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // by starting parity
     int graph_steps = 32;
     int graph_launches = 32;  // kernels of a captured graph
+    // a graph of the caller's holds launches of this handle: its nodes carry
+    // the buffer they read, so from then on n steps swap the buffers as often
+    // as n launches of one step would (modulo 2), and the graph can be
+    // replayed after any even number of further steps
+    bool captured = false;
     int tune_variant = LBM_KERNEL_AUTO;  // the kernel_variant the handle was created with
     // tensor maps (loads, stores) of the population arena for the single-pass
     // TMA kernel (one lattice, or a batch in one row space; rows at least a box
@@ -1175,19 +1180,28 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     int rc = direct ? check_status_async(h) : fault_code(h);
     if (rc) return rc;
     int64_t left = nsteps;
+    if (!direct && left > 0) h->captured = true;
     // resident lattices: from two steps on (one step is one tile-kernel launch;
-    // a resident one costs about 3 us beside its steps)
-    if (direct && h->res_grid && left >= 2 && !h->prof && !h->starve) {
-        while (left >= 2) {
+    // a resident one costs about 3 us beside its steps).  A launch swaps the
+    // buffers once, so a captured handle's launches take odd numbers of steps.
+    if (direct && h->res_grid && !h->prof && !h->starve) {
+        while (left >= (h->captured ? 3 : 2)) {
             // at most 2^14 steps a launch (a fraction of a second)
-            const int n = (int)std::min<int64_t>(left, left == (1 << 14) + 1 ? 1 << 13 : 1 << 14);
+            int n = (int)std::min<int64_t>(left, left == (1 << 14) + 1 ? 1 << 13 : 1 << 14);
+            if (h->captured && !(n & 1)) --n;
             rc = launch_resident_steps(h, n);
             if (rc == LBM_PENDING) break;
             if (rc) return rc;
             left -= n;
         }
     }
-    while (direct && !h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps) {
+    // launches of two steps; they too swap the buffers once, so a captured
+    // handle takes an even number of them
+    int64_t twos = h->path == PATH_PAIRS && direct ? (left - (h->starve ? 1 : 0)) / 2 : 0;
+    if (h->captured) twos &= ~(int64_t)1;
+    const int64_t graph_twos = h->path == PATH_PAIRS ? h->graph_steps / 2 : 0;  // in one graph
+    while (direct && !h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps &&
+           twos >= graph_twos) {
         if (!h->graph[h->parity]) {
             rc = capture_graph(h);
             if (rc) return rc;
@@ -1195,15 +1209,17 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
         CK(h, cudaGraphLaunch(h->graph[h->parity], h->stream));
         h->launches += h->graph_launches;
         left -= h->graph_steps;
+        twos -= graph_twos;
         // an even number of steps, but half as many launches of two
-        if (h->path == PATH_PAIRS && (h->graph_launches & 1)) h->parity ^= 1;
+        if (graph_twos & 1) h->parity ^= 1;
     }
     while (left > 0) {
-        const bool two = h->path == PATH_PAIRS && direct && left >= 2 && !h->starve;
+        const bool two = twos > 0 && !h->starve;
         rc = two ? launch_two_steps(h, h->parity) : launch_step(h, h->parity);
         if (rc) return rc;
         h->parity ^= 1;
         left -= two ? 2 : 1;
+        twos -= two;
     }
     if (direct && !h->status_pending) {
         CK(h, cudaMemcpyAsync(h->status_host, h->status, h->lat.size() * sizeof(uint32_t),

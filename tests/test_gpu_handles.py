@@ -87,3 +87,28 @@ def test_captured_steps_are_single_launches(P, shape, storage, kw):
         got = P.lbm_moments(h, 0)
         P.lbm_destroy(h)
         _same(got, _tile_run(P, d, f, warm + 3 * 34 + 1))
+
+
+@pytest.mark.parametrize("shape,storage", KINDS)
+@pytest.mark.parametrize("kw", [{}, {"graph_steps": 2}, {"graph_steps": -1}])
+def test_replays_alternate_with_direct_steps(P, shape, storage, kw):
+    # a graph of two steps is good for as long as an even number of other
+    # steps lies between its replays, whichever launches took those
+    d, f = P.lbm_desc_default(*shape, T=0.8, storage=storage), _field(*shape)
+    for warm in (1, 2):
+        h = P.lbm_create(d, **kw)
+        P.lbm_init(h, 0, f)
+        P.lbm_step(h, warm)
+        g = _capture(P, h, 2)
+        steps = warm
+        # (a resident launch takes at most 2^14 steps)
+        long = (16386, 2**14 + 1, 1) if shape == (64, 50) and not kw else ()
+        for direct in ((), (4,), (2,), (), (33, 33), (64,), (2, 4), (3, 1), (66,), (130,), long):
+            for n in direct:
+                P.lbm_step(h, n)
+            _replay(h, g)
+            steps += sum(direct) + 2
+        P.lbm_step(h, 7)
+        got = P.lbm_moments(h, 0)
+        P.lbm_destroy(h)
+        _same(got, _tile_run(P, d, f, steps + 7))
