@@ -53,7 +53,10 @@ struct PassCfg {
 enum StepPath { PATH_TILES, PATH_ROWS, PATH_PAIRS };
 struct TuneVal {
     PassCfg pass[2];
-    StepPath path = PATH_TILES;
+    // by collision (LBM_COLL_*), where a row kernel was timed beside the tiles:
+    // a handle without row items has no say in the others'
+    bool timed[2] = {false, false};
+    StepPath path[2] = {PATH_TILES, PATH_TILES};
 };
 
 // One pass of the step (0: psi, 1: force + collision + stream): its kernel
@@ -1058,8 +1061,8 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         auto it = g_tune_cache.find(k);
         if (it != g_tune_cache.end() && !(opts && (opts->tile_x || opts->tile_y))) {
             for (int q = 0; q < 2; ++q) cfg[q] = it->second.pass[q];
-            tuned = true;
-            tuned_path = it->second.path;
+            tuned = it->second.timed[h->collision];
+            tuned_path = it->second.path[h->collision];
         }
     }
     if (cfg[1].variant == LBM_KERNEL_TMA &&
@@ -1446,7 +1449,8 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
     h->prof = false;
     const int64_t launches0 = h->launches;
     int rc = LBM_OK;
-    TuneVal best_cfg{};
+    PassCfg best_cfg[2];
+    bool timed = false;  // a row kernel, against the tile kernel
     // Each pass is tuned on its own.  Trial launches read population buffer
     // `parity` and write psi or the other buffer only, so repeating them
     // leaves the state unchanged; the collision trials run on the psi of
@@ -1502,7 +1506,7 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
         h->pass[k].spt = bc.spt;
         rc = build_tiles(h, k, bc.tx, bc.ty);
         h->pass[k].grid = bc.grid;
-        best_cfg.pass[k] = bc;
+        best_cfg[k] = bc;
         if (k == 1 && h->items && rc == LBM_OK) {
             // the row kernel against the best tile kernel, per step
             const StepPath row = h->f16 ? PATH_ROWS : PATH_PAIRS;
@@ -1516,7 +1520,7 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
             float ms = 0.f;
             cudaEventElapsedTime(&ms, ea, eb);
             if (ms < best * (row == PATH_PAIRS ? 2.f : 1.f)) h->path = row;
-            best_cfg.path = h->path;
+            timed = true;
         }
     }
     cudaEventDestroy(ea);
@@ -1529,7 +1533,12 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     TuneKey key{h->device, h->storage, h->eos, h->tune_variant * 4 + h->schedule,
                 (int64_t)std::log2((double)h->sites), (int64_t)std::log2((double)h->lat.size())};
-    g_tune_cache[key] = best_cfg;
+    TuneVal& v = g_tune_cache[key];
+    for (int k = 0; k < 2; ++k) v.pass[k] = best_cfg[k];
+    if (timed) {
+        v.timed[h->collision] = true;
+        v.path[h->collision] = h->path;
+    }
     return LBM_OK;
 }
 

@@ -112,3 +112,26 @@ def test_replays_alternate_with_direct_steps(P, shape, storage, kw):
         got = P.lbm_moments(h, 0)
         P.lbm_destroy(h)
         _same(got, _tile_run(P, d, f, steps + 7))
+
+
+# ------------------------------------------------------------ tuned choices
+def test_autotune_leaves_the_paths_it_did_not_time(P):
+    # two lattices tuned on a handle that has no row kernel (resident) and a
+    # larger pair of the same size class: that one keeps its two-step launches
+    small = [P.lbm_desc_default(520, 520, T=0.8)] * 2
+    large = [P.lbm_desc_default(700, 720, T=0.8)] * 2
+    h = P.lbm_create(small)
+    for i in range(2):
+        P.lbm_init(h, i, _field(520, 520, i))
+    l0 = P.lbm_launch_count(h)
+    P.lbm_step(h, 10)
+    assert P.lbm_launch_count(h) - l0 == 1
+    P.lbm_autotune(h, 1)
+    P.lbm_destroy(h)
+    h = P.lbm_create(large)
+    for i in range(2):
+        P.lbm_init(h, i, _field(700, 720, i))
+    l0 = P.lbm_launch_count(h)
+    P.lbm_step(h, 10)
+    assert P.lbm_launch_count(h) - l0 == 5
+    P.lbm_destroy(h)
