@@ -63,8 +63,9 @@ def _replay(h, g):
 
 
 # ------------------------------------------------ graphs captured by the caller
-# (sites, storage): resident, two steps a launch, one step a launch on rows
-KINDS = [((64, 50), 1), ((1100, 901), 1), ((1100, 901), 2)]
+# (sites, storage): resident, two steps a launch, resident in FP16 storage
+# only, one step a launch on rows
+KINDS = [((64, 50), 1), ((1100, 901), 1), ((1100, 901), 2), ((1300, 1201), 2)]
 
 
 @pytest.mark.parametrize("shape,storage", KINDS)
