@@ -246,9 +246,10 @@ typedef struct {
 } lbm_kernel_stat;
 
 /* Waits, then reads the per-kernel records since lbm_profile(h, 1) into
- * out[0..max), returning the number of kernels in *n: the psi pass, the
- * single-pass (or collision) step and, where it ran, the launch of two
- * steps.  While recording, no launch takes more than two steps. */
+ * out[0..max), returning in *n how many it wrote (at most max; with out NULL,
+ * how many there are): the psi pass, the single-pass (or collision) step and,
+ * where it ran, the launch of two steps.  While recording, no launch takes
+ * more than two steps. */
 int lbm_profile_read(lbm_handle* h, lbm_kernel_stat* out, int32_t max, int32_t* n);
 
 /* Number of kernels this handle has launched so far (graph replays count

@@ -1396,7 +1396,7 @@ static int lbm_profile_read_body(lbm_handle* h, lbm_kernel_stat* out, int32_t ma
         out[k].total_ms = h->rec[k].total_ms;
         out[k].bytes_per_launch = h->rec[k].bytes;
     }
-    *n = cnt;
+    *n = out ? std::min(cnt, std::max(max, 0)) : cnt;
     return LBM_OK;
 }
 

@@ -136,3 +136,22 @@ def test_autotune_leaves_the_paths_it_did_not_time(P):
     P.lbm_step(h, 10)
     assert P.lbm_launch_count(h) - l0 == 5
     P.lbm_destroy(h)
+
+
+# ------------------------------------------------------------------ records
+def test_profile_read_gives_at_most_max_records(P):
+    import ctypes
+
+    h = P.lbm_create(P.lbm_desc_default(1100, 901, T=0.8))
+    P.lbm_init(h, 0, _field(1100, 901))
+    P.lbm_profile(h, True)
+    P.lbm_step(h, 5)
+    for size in (0, 1, 2, 3, 8):
+        arr = (P.KernelStat * 9)()
+        arr[size].launches = -7
+        n = ctypes.c_int32(-1)
+        assert P.load().lbm_profile_read(h.ptr, arr, size, ctypes.byref(n)) == 0
+        assert n.value == min(size, 3) and arr[size].launches == -7
+    n = ctypes.c_int32(-1)
+    assert P.load().lbm_profile_read(h.ptr, None, 0, ctypes.byref(n)) == 0 and n.value == 3
+    P.lbm_destroy(h)
