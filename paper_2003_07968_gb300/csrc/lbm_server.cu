@@ -1053,12 +1053,15 @@ static int lbm_server_create_body(const lbm_server_opts* opts, lbm_server** out)
         S->pass[1].spt = kPassDefaults[1].spt;
     }
     // the row kernels, FP32 storage two steps a launch (where the tallest
-    // request's rows fit their 32-bit offsets)
+    // request's rows fit their 32-bit offsets).  Chunks of one step in FP32
+    // storage stay on the tile kernel: 200 lattices of 64^2 .. 512^2 in such
+    // chunks keep the GPU busy for 20.6 ms on it and for 24.3 on k_rows (in
+    // chunks of two steps 18.7, on k_rows2, against 20.5).
     LatDev tallest{};
     tallest.pitch = (int32_t)S->pitch;
     tallest.ny = (int32_t)std::min<int64_t>(o.max_request_sites / 2, S->row_cap);
     S->rows = S->tma && o.kernel_variant == LBM_KERNEL_AUTO && o.eos_precision == LBM_EOS_DF &&
-              !(o.tile_x || o.tile_y) && rows_fit(tallest, S->es);
+              !(o.tile_x || o.tile_y) && (S->f16 || o.chunk_steps > 1) && rows_fit(tallest, S->es);
     S->pairs = S->rows && !S->f16;
     S->st.arena_bytes = (int64_t)o.arena_bytes;
     try {

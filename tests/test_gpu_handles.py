@@ -155,3 +155,39 @@ def test_profile_read_gives_at_most_max_records(P):
     n = ctypes.c_int32(-1)
     assert P.load().lbm_profile_read(h.ptr, None, 0, ctypes.byref(n)) == 0 and n.value == 3
     P.lbm_destroy(h)
+
+
+# ------------------------------------------------------------------ the server
+def test_server_chunks_of_one_step_keep_the_tile_kernels_speed(P):
+    # FP32 requests in chunks of one step gain nothing from the row kernels;
+    # bitwise the same results, and the GPU no busier than on the tile kernel
+    # (8 % for the noise of a busy time of some 20 ms; k_rows took 18 % more)
+    import time
+
+    rng = np.random.default_rng(3)
+    sizes = [tuple(int(v) for v in rng.integers(64, 513, 2)) for _ in range(120)]
+    fields = [synth.droplet(nx, ny, 0.3 * min(nx, ny), 0.8) for nx, ny in sizes]
+    busy, results = {}, {}
+    for variant in (P.LBM_KERNEL_AUTO, P.LBM_KERNEL_TMA) * 3:
+        srv = P.lbm_server_create(P.lbm_server_opts_default(
+            chunk_steps=1, with_velocity=0, kernel_variant=variant))
+        tickets = [P.lbm_submit(srv, P.lbm_desc_default(nx, ny, T=0.8), f, 60)
+                   for (nx, ny), f in zip(sizes, fields)]
+        got = {}
+        t0 = time.time()
+        while len(got) < len(tickets):
+            for t in tickets:
+                if t not in got:
+                    r = P.lbm_poll(srv, t, u=False)
+                    if r is not None:
+                        got[t] = r["rho"]
+            assert time.time() - t0 < 60
+            time.sleep(0.001)
+        st = P.lbm_server_get_stats(srv)
+        P.lbm_server_destroy(srv)
+        busy.setdefault(variant, []).append(st["busy_s"])
+        results[variant] = [got[t] for t in tickets]
+    for a, b in zip(results[P.LBM_KERNEL_AUTO], results[P.LBM_KERNEL_TMA]):
+        assert np.array_equal(a, b)
+    print(busy)
+    assert min(busy[P.LBM_KERNEL_AUTO]) <= 1.08 * min(busy[P.LBM_KERNEL_TMA])
