@@ -122,7 +122,11 @@ struct lbm_handle {
     cudaStream_t side = nullptr;  // copies of lbm_moments results, beside the kernels
     cudaEvent_t chunk_ev[5] = {};
     int64_t device_bytes = 0;
-    // host side
+    // host side: lists on their way to the device.  A copy from pageable memory
+    // may read it after the call returns, so they are kept until the stream has
+    // been waited for (the end of lbm_create, each trial of lbm_autotune).
+    std::vector<std::vector<int4>> sent;
+    std::vector<ResTile> sent_tiles;
     double* scan_host = nullptr;      // pinned: a device result (lbm_init's scan, the mass)
     uint32_t* status_host = nullptr;  // ... and the fault words after it
     cudaEvent_t status_ev = nullptr;
@@ -254,11 +258,11 @@ int build_tiles(lbm_handle* h, int k, int tx, int ty) {
         }
         P.cap = bytes;
     }
-    // (a copy from pageable memory has read it when the call returns)
-    CK(h, cudaMemcpyAsync(P.tiles, t.data(), bytes, cudaMemcpyHostToDevice, h->stream));
     P.tx = tx;
     P.ty = ty;
     P.ntiles = (int)t.size();
+    h->sent.push_back(std::move(t));
+    CK(h, cudaMemcpyAsync(P.tiles, h->sent.back().data(), bytes, cudaMemcpyHostToDevice, h->stream));
     return LBM_OK;
 }
 
@@ -347,7 +351,7 @@ int make_resident(lbm_handle* h) {
     int coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess || !coop)
         return LBM_OK;
-    const ResPlan P = plan_resident(h->lat, std::min(2 * h->sm_count, kResBlocks), h->f16 ? 2 : 4);
+    ResPlan P = plan_resident(h->lat, std::min(2 * h->sm_count, kResBlocks), h->f16 ? 2 : 4);
     if (P.tiles.empty()) return LBM_OK;
     const int per_sm =
         resident_blocks_per_sm(h->f16, h->collision == LBM_COLL_MRT, h->lat.size() == 1);
@@ -357,8 +361,8 @@ int make_resident(lbm_handle* h) {
     h->res_bytes = res_epoch_off(h) + h->res_grid * sizeof(uint32_t);
     h->res = dev_alloc(h, h->res_bytes);
     if (!h->res) return LBM_ERR_OOM;
-    // (a copy from pageable memory has read it when the call returns)
-    CK(h, cudaMemcpyAsync(h->res, P.tiles.data(), P.tiles.size() * sizeof(ResTile),
+    h->sent_tiles = std::move(P.tiles);
+    CK(h, cudaMemcpyAsync(h->res, h->sent_tiles.data(), h->sent_tiles.size() * sizeof(ResTile),
                           cudaMemcpyHostToDevice, h->stream));
     return LBM_OK;
 }
@@ -377,8 +381,10 @@ int make_items(lbm_handle* h) {
     h->items_bytes = t.size() * sizeof(int4);
     h->items = (int4*)dev_alloc(h, h->items_bytes);
     if (!h->items) return LBM_ERR_OOM;
-    CK(h, cudaMemcpyAsync(h->items, t.data(), h->items_bytes, cudaMemcpyHostToDevice, h->stream));
     h->n_items = (int)t.size();
+    h->sent.push_back(std::move(t));
+    CK(h, cudaMemcpyAsync(h->items, h->sent.back().data(), h->items_bytes, cudaMemcpyHostToDevice,
+                          h->stream));
     return LBM_OK;
 }
 
@@ -1109,6 +1115,8 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
     h->rec[1].bytes = (double)h->sites * (h->schedule == LBM_SCHED_FUSED ? 18.0 * es
                                                                         : 18.0 * es + 4.0);
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) return fail(LBM_ERR_CUDA);
+    h->sent.clear();
+    std::vector<ResTile>().swap(h->sent_tiles);
     *out = h;
     return LBM_OK;
 }
@@ -1493,6 +1501,7 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
                 cudaEventRecord(eb, h->stream);
                 if (e == cudaSuccess) e = cudaEventSynchronize(eb);
                 if (e != cudaSuccess) { rc = cuda_fail(h, e, "autotune"); break; }
+                h->sent.clear();
                 float ms = 0.f;
                 cudaEventElapsedTime(&ms, ea, eb);
                 if (ms < best) {
@@ -1530,6 +1539,7 @@ static int lbm_autotune_body(lbm_handle* h, int32_t repeats) {
     if (rc) return rc;
     rc = sync_status(h);
     if (rc) return rc;
+    h->sent.clear();
     std::lock_guard<std::mutex> lk(g_tune_mu);
     TuneKey key{h->device, h->storage, h->eos, h->tune_variant * 4 + h->schedule,
                 (int64_t)std::log2((double)h->sites), (int64_t)std::log2((double)h->lat.size())};

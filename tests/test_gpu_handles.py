@@ -191,3 +191,22 @@ def test_server_chunks_of_one_step_keep_the_tile_kernels_speed(P):
         assert np.array_equal(a, b)
     print(busy)
     assert min(busy[P.LBM_KERNEL_AUTO]) <= 1.08 * min(busy[P.LBM_KERNEL_TMA])
+
+
+# ---------------------------------------------------- lists sent to the device
+@pytest.mark.parametrize("shape,storage", KINDS)
+def test_create_on_a_busy_stream(P, shape, storage):
+    # the tile and item lists reach the device after lbm_create has queued
+    # their copies behind the caller's work, and stay in host memory until then
+    import torch
+
+    d, f = P.lbm_desc_default(*shape, T=0.8, storage=storage), _field(*shape)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        torch.cuda._sleep(200_000_000)  # about 0.1 s
+    h = P.lbm_create(d, stream=stream)
+    P.lbm_init(h, 0, f)
+    P.lbm_step(h, 5)
+    got = P.lbm_moments(h, 0)
+    P.lbm_destroy(h)
+    _same(got, _tile_run(P, d, f, 5))
