@@ -595,10 +595,11 @@ int sync_status(lbm_handle* h, bool copied = false) {
 }
 
 // The device's address of n host doubles that kernels may write themselves:
-// page-locked (both ends), on a device that reaches host memory coherently.
-// Null where a copy has to bring the field.
+// page-locked (both ends) and at a multiple of eight bytes, on a device that
+// reaches host memory coherently.  Null where a copy, which takes any address,
+// has to bring the field.
 double* host_direct(const lbm_handle* h, double* p, size_t n) {
-    if (!h->host_access || !p) return nullptr;
+    if (!h->host_access || !p || reinterpret_cast<uintptr_t>(p) % sizeof(double)) return nullptr;
     cudaPointerAttributes a{}, b{};
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess ||
         cudaPointerGetAttributes(&b, p + n - 1) != cudaSuccess) {

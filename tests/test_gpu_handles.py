@@ -210,3 +210,29 @@ def test_create_on_a_busy_stream(P, shape, storage):
     got = P.lbm_moments(h, 0)
     P.lbm_destroy(h)
     _same(got, _tile_run(P, d, f, 5))
+
+
+# ------------------------------------------------------------ fields read back
+@pytest.mark.parametrize("offset", [1, 2, 4, 7])
+def test_page_locked_arrays_at_any_address(P, offset):
+    # a packed record may hold a field at an address that is no multiple of
+    # eight: such an array is filled by a copy, as pageable ones are
+    import torch
+
+    nx, ny = 64, 50
+    h = P.lbm_create(P.lbm_desc_default(nx, ny, T=0.8))
+    P.lbm_init(h, 0, _field(nx, ny))
+    P.lbm_step(h, 4)
+    want = P.lbm_moments(h, 0)
+    raw = torch.zeros(8 * nx * ny + 16, dtype=torch.uint8, pin_memory=True).numpy()
+    got = {}
+    for key in ("rho", "ux", "uy"):
+        raw[:] = 255
+        out = raw[offset:offset + 8 * nx * ny].view(np.float64).reshape(ny, nx)
+        P.lbm_moments(h, 0, rho=key == "rho", u=key != "rho", mass=False,
+                      out={**{k: np.empty((ny, nx)) for k in ("ux", "uy")}, key: out})
+        got[key] = out.copy()
+        assert np.all(raw[:offset] == 255) and np.all(raw[offset + 8 * nx * ny:] == 255)
+    got["mass"] = want["mass"]
+    P.lbm_destroy(h)
+    _same(got, want)
