@@ -65,21 +65,37 @@ constexpr size_t pair_smem(int es) { return (size_t)kPairs * kPairDepth * 9 * 64
 // in one wave of 53 rows, 53-60 in items of 32 to 64; 3000^2 106 us in two
 // waves of 67, 112-144 in items of 48 to 192; 512 lattices 726 us in items of
 // 96 rows, 793 in four waves of 230.
+//
+// Lattices of few rows make an item however low it is, and beside many of them
+// no height, or only a large one, keeps the count of items within the waves: a
+// taller lattice's items would then run on long after all others.  So the
+// height is at most twice an even share of the rows, and beyond that the one
+// at which the lattices' work, not their items, fills the waves.  2000 lattices
+// of 16^2 and one of 512^2: items of 512 rows 288 us a step, of 31 43 (tile
+// kernel 78); 5000 of 32^2 and one of 2048^2: 1221 and 200 us (478).
 inline int pair_item_height(const std::vector<LatDev>& lats, int64_t pairs) {
     int64_t units = 0, most = 0;
     for (const LatDev& L : lats) {
         units += (int64_t)strip_count(L.nx, kPairCols) * L.ny;
         most = std::max<int64_t>(most, L.ny);
     }
+    const bool one = lats.size() == 1;
     int64_t waves = std::max<int64_t>(1, (units + 36 * pairs) / (72 * pairs));
-    if (lats.size() == 1) waves = std::min<int64_t>(waves, 4);
-    int64_t h = std::max<int64_t>(4, units / (waves * pairs));
-    for (; h < most; ++h) {
-        int64_t n = 0;
+    if (one) waves = std::min<int64_t>(waves, 4);
+    const int64_t share = std::max<int64_t>(4, units / (waves * pairs));
+    for (int64_t h = share; h < most && (one || h <= 2 * share); ++h) {
+        int64_t n = 0;  // items
         for (const LatDev& L : lats) n += strip_count(L.nx, kPairCols) * ((L.ny + h - 1) / h);
-        if (n <= waves * pairs) break;
+        if (n <= waves * pairs) return (int)h;
     }
-    return (int)std::min<int64_t>(h, most);
+    if (one || 2 * share >= most) return (int)most;
+    for (int64_t h = share; h < most; ++h) {
+        int64_t rows = 0;  // a lattice below h counts with its rows, others with whole items
+        for (const LatDev& L : lats)
+            rows += strip_count(L.nx, kPairCols) * (L.ny < h ? L.ny : (L.ny + h - 1) / h * h);
+        if (rows <= waves * pairs * h) return (int)h;
+    }
+    return (int)most;
 }
 // 32-bit offsets of k_rows2: a lattice's rows in a plane take less than 4 GB
 inline bool rows_fit(const LatDev& L, int es) {
