@@ -291,7 +291,8 @@ int lbm_autotune(lbm_handle* h, int32_t repeats);
  * sites stay below a target; a
  * chunk runs each lattice for min(k, its remaining steps), where k is the
  * number of steps that fills about chunk_ms of GPU time at the throughput
- * measured on earlier chunks (CUDA event timings), capped at chunk_steps.
+ * measured on earlier chunks (CUDA event timings), capped at chunk_steps
+ * (and an even number, 2 or more, where two steps go in a launch).
  * Short chunks keep admission and completion close to the request's own
  * work when the GPU is lightly loaded.  The
  * worker keeps two chunks in flight: new requests' fields are uploaded

@@ -236,3 +236,38 @@ def test_page_locked_arrays_at_any_address(P, offset):
     got["mass"] = want["mass"]
     P.lbm_destroy(h)
     _same(got, want)
+
+
+def test_server_chunks_of_little_time_keep_the_tile_kernels_speed(P):
+    # chunk_ms far below a step's time: FP32 requests still advance two steps
+    # a launch rather than one at a time on k_rows, so the GPU is no busier per
+    # step than on the tile kernel (8 % for noise, as above), bitwise the same
+    import time
+
+    rng = np.random.default_rng(4)
+    sizes = [tuple(int(v) for v in rng.integers(64, 513, 2)) for _ in range(120)]
+    fields = [synth.droplet(nx, ny, 0.3 * min(nx, ny), 0.8) for nx, ny in sizes]
+    busy, results = {}, {}
+    for variant in (P.LBM_KERNEL_AUTO, P.LBM_KERNEL_TMA) * 3:
+        srv = P.lbm_server_create(P.lbm_server_opts_default(
+            chunk_ms=1e-4, with_velocity=0, kernel_variant=variant))
+        tickets = [P.lbm_submit(srv, P.lbm_desc_default(nx, ny, T=0.8), f, 60 + k % 3)
+                   for k, ((nx, ny), f) in enumerate(zip(sizes, fields))]
+        got = {}
+        t0 = time.time()
+        while len(got) < len(tickets):
+            for t in tickets:
+                if t not in got:
+                    r = P.lbm_poll(srv, t, u=False)
+                    if r is not None:
+                        got[t] = r["rho"]
+            assert time.time() - t0 < 60
+            time.sleep(0.001)
+        st = P.lbm_server_get_stats(srv)
+        P.lbm_server_destroy(srv)
+        busy.setdefault(variant, []).append(st["busy_s"])
+        results[variant] = [got[t] for t in tickets]
+    for a, b in zip(results[P.LBM_KERNEL_AUTO], results[P.LBM_KERNEL_TMA]):
+        assert np.array_equal(a, b)
+    print(busy)
+    assert min(busy[P.LBM_KERNEL_AUTO]) <= 1.08 * min(busy[P.LBM_KERNEL_TMA])
