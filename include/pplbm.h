@@ -431,6 +431,18 @@ int lbm_mass_noalloc(const float* values, int64_t count, double offset, double* 
  * range). */
 int lbm_inject_copy_timeout(lbm_handle* h, int32_t tile);
 
+/* The same of the launches whose warps or blocks wait for one another: the
+ * next launch of many steps (its tiles' packets) or of two steps (the rows
+ * one warp hands to another), whichever the handle makes.  What tile or item
+ * `item` (counted from 0, as the launch has them) sends is never counted as
+ * arrived: its neighbours' waits run out after the same short limit (a tile
+ * that is its lattice's only one is its own neighbour and notices nothing),
+ * theirs in turn, and every block and warp leaves.  lbm_sync reports
+ * LBM_ERR_TIMEOUT; lbm_init clears the fault.  Stays armed until such a launch
+ * comes; no CUDA graph replays it.  Errors: LBM_ERR_ARG (no handle, none of
+ * its launches is of that kind, item out of range). */
+int lbm_inject_wait_timeout(lbm_handle* h, int32_t item);
+
 /* The reciprocal and square root of the step kernels (the hardware
  * approximations, each refined by one Newton-Raphson step on the paired FP32
  * pipe; used by the float-float EOS, Eqs. DED and CSEOS, and by the velocity of

@@ -141,6 +141,7 @@ SIGNATURES = {
     "lbm_info": (ctypes.c_int, [_vp, ctypes.POINTER(Info)]),
     "lbm_autotune": (ctypes.c_int, [_vp, ctypes.c_int32]),
     "lbm_inject_copy_timeout": (ctypes.c_int, [_vp, ctypes.c_int32]),
+    "lbm_inject_wait_timeout": (ctypes.c_int, [_vp, ctypes.c_int32]),
     "lbm_selfcheck": (ctypes.c_int, [ctypes.c_char_p, ctypes.c_int32]),
     "lbm_selfcheck_arith": (ctypes.c_int, [ctypes.POINTER(ctypes.c_float), ctypes.c_int64,
                                            ctypes.POINTER(ctypes.c_float),
@@ -416,6 +417,11 @@ def lbm_selfcheck() -> tuple[int, str]:
 def lbm_inject_copy_timeout(h: Handle, tile: int) -> None:
     """Arm the failure-detection test of the single pass for the next step."""
     _check(load().lbm_inject_copy_timeout(h.ptr, int(tile)), "lbm_inject_copy_timeout", h)
+
+
+def lbm_inject_wait_timeout(h: Handle, item: int) -> None:
+    """Arm the failure-detection test of the next launch of many or of two steps."""
+    _check(load().lbm_inject_wait_timeout(h.ptr, int(item)), "lbm_inject_wait_timeout", h)
 
 
 def lbm_selfcheck_psi(desc: LatticeDesc, rho) -> tuple[np.ndarray, np.ndarray]:

@@ -131,7 +131,8 @@ struct StepArgs {
     int step;
     int last_only = 0;  // k_rows: only lattices whose quota ends with this step
     // failure-detection test: tile + 1 whose staging copy the single pass
-    // skips, so that the consumers' bounded wait for it runs out (0: none)
+    // skips, or item + 1 whose first warp's rows k_rows2 never counts as handed
+    // over, so that the bounded waits for them run out (0: none)
     int starve = 0;
     // clock budget of the single pass's waits (SM cycles): kWaitBudgetCycles,
     // or kTestWaitBudgetCycles in the launch that carries an armed test.  A

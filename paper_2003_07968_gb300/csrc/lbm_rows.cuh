@@ -318,7 +318,12 @@ __global__ void __launch_bounds__(64 * kPairs, 2)
         on = !a.quota || a.step + 2 <= __ldg(&a.quota[tl.x]);
     }
     if (w < kPairs && lane == 0) {
-        for (int k = 0; k < 2 * kPairDepth; ++k) mbar_init(&full[k], 1);
+        // (failure-detection test: an armed item's rows never count as handed over)
+        const uint32_t arrivals = a.starve == t + 1 ? 2 : 1;
+        for (int k = 0; k < kPairDepth; ++k) {
+            mbar_init(&full[k], arrivals);
+            mbar_init(&empty[k], 1);
+        }
         mbar_fence_init();
     }
     if (!ONE && w < kPairs && on)

@@ -132,6 +132,7 @@ struct lbm_handle {
     cudaEvent_t status_ev = nullptr;
     bool status_pending = false;
     int32_t starve = 0;        // armed failure-detection test (tile + 1), for one launch
+    int32_t starve_item = 0;   // the same of a launch of many or of two steps (tile or item + 1)
     int numeric_lattice = -1;  // first lattice with a device fault bit
     uint32_t fault_bits = 0;   // OR of the device fault bits seen
     int sm_count = 0;
@@ -390,10 +391,12 @@ int make_items(lbm_handle* h) {
 
 // The row kernel over the handle's items, from buffer `parity` to the other:
 // one step (FP16 storage) or two (FP32).
-cudaError_t launch_row_steps(lbm_handle* h, int parity) {
+cudaError_t launch_row_steps(lbm_handle* h, int parity, int32_t starve = 0) {
     StepArgs a = step_args(h, parity, 1);
     a.tiles = h->items;
     a.ntiles = h->n_items;
+    a.starve = starve;
+    if (starve) a.wait_cycles = kTestWaitBudgetCycles;
     return (h->f16 ? launch_rows : launch_pairs)(h->f16, h->collision == LBM_COLL_MRT, a,
                                                  h->lat.size() == 1 ? &h->lat[0] : nullptr, h->stream);
 }
@@ -414,6 +417,13 @@ int launch_resident_steps(lbm_handle* h, int nsteps) {
     m.epoch = reinterpret_cast<uint32_t*>(static_cast<char*>(h->res) + res_epoch_off(h));
     m.slot = h->res_slot;
     m.nsteps = nsteps;
+    if (h->starve_item) {
+        // an armed failure-detection test: the tile's packets carry numbers that
+        // none of its neighbours waits for (lbm_init clears the epochs)
+        CK(h, cudaMemsetAsync(m.epoch + (h->starve_item - 1), 0x80, sizeof(uint32_t), h->stream));
+        m.a.wait_cycles = kTestWaitBudgetCycles;
+        h->starve_item = 0;
+    }
     Flights& F = flights_of(h->device);
     std::lock_guard<std::mutex> lk(F.mu);
     auto mine = F.list.end();
@@ -516,7 +526,9 @@ int launch_two_steps(lbm_handle* h, int p) {
         e2 = take_event(h);
         CK(h, cudaEventRecord(e1, h->stream));
     }
-    CK(h, launch_row_steps(h, p));
+    const int32_t starve = h->starve_item;  // goes into this launch only
+    h->starve_item = 0;
+    CK(h, launch_row_steps(h, p, starve));
     if (h->prof) {
         CK(h, cudaEventRecord(e2, h->stream));
         h->rec[2].pending.emplace_back(e1, e2);
@@ -1212,8 +1224,8 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     int64_t twos = h->path == PATH_PAIRS && direct ? (left - (h->starve ? 1 : 0)) / 2 : 0;
     if (h->captured) twos &= ~(int64_t)1;
     const int64_t graph_twos = h->path == PATH_PAIRS ? h->graph_steps / 2 : 0;  // in one graph
-    while (direct && !h->prof && !h->starve && h->graph_steps > 0 && left >= h->graph_steps &&
-           twos >= graph_twos) {
+    while (direct && !h->prof && !h->starve && !h->starve_item && h->graph_steps > 0 &&
+           left >= h->graph_steps && twos >= graph_twos) {
         if (!h->graph[h->parity]) {
             rc = capture_graph(h);
             if (rc) return rc;
@@ -1569,6 +1581,18 @@ static int lbm_inject_copy_timeout_body(lbm_handle* h, int32_t tile) {
 
 int lbm_inject_copy_timeout(lbm_handle* h, int32_t tile) {
     return guarded([&] { return lbm_inject_copy_timeout_body(h, tile); });
+}
+
+static int lbm_inject_wait_timeout_body(lbm_handle* h, int32_t item) {
+    if (!h) return LBM_ERR_ARG;
+    const int n = h->res_grid ? h->res_grid : h->path == PATH_PAIRS ? h->n_items : 0;
+    if (item < 0 || item >= n) return LBM_ERR_ARG;
+    h->starve_item = item + 1;  // the next launch of many or of two steps; no graph replays it
+    return LBM_OK;
+}
+
+int lbm_inject_wait_timeout(lbm_handle* h, int32_t item) {
+    return guarded([&] { return lbm_inject_wait_timeout_body(h, item); });
 }
 
 static int lbm_selfcheck_arith_body(const float* x, int64_t n, float* rcp, float* sq) {

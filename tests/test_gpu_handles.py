@@ -238,6 +238,60 @@ def test_page_locked_arrays_at_any_address(P, offset):
     _same(got, want)
 
 
+# ------------------------------------------------------------- bounded waits
+# lattices (the first is the one that fails), storage, collision, armed item:
+# many steps a launch (one lattice and a batch, each storage, MRT), two steps
+WAITS = [([(64, 50)], 1, 0, 0), ([(203, 77)], 2, 1, 5), ([(64, 64), (61, 100)], 1, 0, 3),
+         ([(1100, 901)], 1, 0, 7), ([(1100, 901)], 1, 1, 0), ([(1100, 901), (61, 300)], 1, 0, 20)]
+
+
+@pytest.mark.parametrize("shapes,storage,mrt,item", WAITS)
+def test_waits_of_the_long_launches_run_out(P, shapes, storage, mrt, item):
+    # what one tile or item sends never counts as arrived: the others' waits
+    # give up after about 0.1 s, every block leaves, lbm_init clears the fault,
+    # and a second lattice of the handle never notices
+    import time
+
+    kw = dict(collision=P.LBM_COLL_MRT, tau=0.7, mrt_rates=[1.0] * 7 + [1.0 / 0.7] * 2) if mrt else {}
+    descs = [P.lbm_desc_default(nx, ny, T=0.8, storage=storage, **kw) for nx, ny in shapes]
+    fields = [_field(nx, ny, k) for k, (nx, ny) in enumerate(shapes)]
+    h = P.lbm_create(descs)
+    for k, f in enumerate(fields):
+        P.lbm_init(h, k, f)
+    P.lbm_step(h, 4)
+    P.lbm_sync(h)
+    with pytest.raises(P.LbmError) as err:
+        P.lbm_inject_wait_timeout(h, 1 << 30)
+    assert err.value.code == P.LBM_ERR_ARG
+    P.lbm_inject_wait_timeout(h, item)
+    P.lbm_step(h, 1)  # one step: not a launch of that kind, the test stays armed
+    P.lbm_sync(h)
+    t0 = time.time()
+    P.lbm_step(h, 6)
+    with pytest.raises(P.LbmError) as err:
+        P.lbm_sync(h)
+    waited = time.time() - t0
+    assert err.value.code == P.LBM_ERR_TIMEOUT and P.lbm_status_detail(h) == 0
+    assert 0.05 < waited < 1.5
+    with pytest.raises(P.LbmError):
+        P.lbm_step(h, 2)
+    P.lbm_init(h, 0, fields[0])
+    P.lbm_step(h, 20)
+    got = [P.lbm_moments(h, k) for k in range(len(shapes))]
+    P.lbm_destroy(h)
+    for k, g in enumerate(got):
+        _same(g, _tile_run(P, descs[k], fields[k], 20 if k == 0 else 31))
+
+
+def test_wait_test_refused_where_no_launch_waits(P):
+    for kw, storage in (({"kernel_variant": P.LBM_KERNEL_TMA}, 1), ({}, 2)):
+        h = P.lbm_create(P.lbm_desc_default(1300, 1201, T=0.8, storage=storage), **kw)
+        with pytest.raises(P.LbmError) as err:
+            P.lbm_inject_wait_timeout(h, 0)
+        P.lbm_destroy(h)
+        assert err.value.code == P.LBM_ERR_ARG
+
+
 def test_server_chunks_of_little_time_keep_the_tile_kernels_speed(P):
     # chunk_ms far below a step's time: FP32 requests still advance two steps
     # a launch rather than one at a time on k_rows, so the GPU is no busier per
