@@ -98,8 +98,8 @@ extern "C" {
                               take over: lattices that fit the SMs' shared
                               memory advance many steps a launch, others in
                               FP32 storage two, in FP16 storage one on a row
-                              kernel (lbm_info names the tile kernel, which
-                              takes the steps that are left)              */
+                              kernel, where their widths suit it (lbm_info
+                              names the tile kernel, which takes the rest) */
 #define LBM_KERNEL_PLAIN 1 /* plain global loads, 1, 2 or 4 sites per thread
                               (with 2 or 4, site pairs share the paired FP32
                               instructions); tile_x a multiple of 32,
@@ -283,8 +283,8 @@ int lbm_autotune(lbm_handle* h, int32_t repeats);
 /* ---- serving: continuous batching --------------------------------------- */
 /* A server keeps many independent lattices (requests) resident in one
  * device arena and steps all of them together: a chunk of steps is a launch
- * per step, or per two steps in FP32 storage, over a list that spans every
- * resident lattice (the same kernels as a batch handle).  Requests are admitted at
+ * per step, or per two steps in FP32 storage where the resident lattices'
+ * widths suit the row kernel, over a list that spans every resident lattice (the same kernels as a batch handle).  Requests are admitted at
  * chunk boundaries, first come first served but skipping any that do not
  * fit yet, whenever a slot and arena space (HBM footprint: both population
  * buffers at the arena's common pitch, plus psi) are free and the resident

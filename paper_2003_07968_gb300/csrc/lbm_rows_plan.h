@@ -97,6 +97,63 @@ inline int pair_item_height(const std::vector<LatDev>& lats, int64_t pairs) {
     }
     return (int)most;
 }
+// ---- row kernel or tile kernel
+// Estimated microseconds of a step on the row kernel of the storage (one: one
+// lattice, by value; else the batch instance) over items of `height` rows, and
+// on the tile kernel the handle has (tensor: the TMA kernel's 32 x 16 tiles;
+// else plain loads).  A warp's rows come one after another, whatever the
+// others do, so a launch lasts as long as its tallest item or its waves of
+// items; what the warps of an SM share (the FP32 pipe) adds a part by the total
+// of rows.  A strip costs its 64 columns even if it holds 32 (a lattice 64
+// columns wide is two such strips and four tiles), which is where the tile
+// kernel wins.  Fitted to 65 shapes in each storage, BGK and MRT, from one
+// lattice to 5000 and 16 k to 17 M sites: nine of ten of the row kernels' times
+// lie within 12 %, of the tile kernels' within 20 % (theirs vary with the pitch).
+inline double rows_us(const std::vector<LatDev>& lats, int height, bool f16, bool mrt, bool one,
+                      int64_t sms) {
+    const int cols = f16 ? kRowCols : kPairCols, halo = f16 ? 3 : 6;
+    const int64_t slots = sms * (f16 ? 4 * kRowWarps : 2 * kPairs);
+    int64_t n = 0, work = 0, tallest = 0;
+    for (const LatDev& L : lats) {
+        const int64_t ns = strip_count(L.nx, cols), nb = (L.ny + height - 1) / height;
+        n += ns * nb;
+        work += ns * (L.ny + halo * nb);
+        tallest = std::max<int64_t>(tallest, (L.ny + nb - 1) / nb + halo);
+    }
+    const double waves = (double)((n + slots - 1) / slots);
+    const double chain = std::max((double)tallest, waves * (double)work / (double)n);
+    const double start = f16 ? (one ? 7.0 : 5.0) : 0.5;
+    const double per_row = f16 ? (one ? 0.3 : 0.09) : (one ? 0.43 : 0.61);
+    const double shared = f16 ? (one ? 1.09 : 1.5) : (one ? 0.35 : 0.25);
+    return start + (chain * per_row + (double)work / (double)slots * shared) *
+                       (mrt ? (one ? 1.17 : 1.12) : 1.0);
+}
+inline double tiles_us(const std::vector<LatDev>& lats, bool mrt, bool tensor) {
+    double us = 0.0;
+    for (const LatDev& L : lats) {
+        const double across = (L.nx + 31) / 32, down = (L.ny + 15) / 16;
+        if (lats.size() == 1)  // a tile cut at the right edge is stored without the TMA
+            us += down * (0.0088 * (L.nx / 32) + 0.0112 * (across - L.nx / 32));
+        else if (tensor)
+            us += 0.009 * across * down;
+        else
+            us += 0.0052 * across * down + 0.0138 / 512.0 * L.nx * L.ny;
+    }
+    return 4.6 + us * (mrt ? 1.1 : 1.0);
+}
+// Whether the row kernel takes the lattices.  Measured per step, tile kernel
+// against row kernel: 310 lattices of 64^2 30 and 60 us (FP16 storage 32 and
+// 42), 400 of 60^2 39 and 59, 1000 of 32^2 26 and 34, one of 64 x 62500 in FP16
+// 84 and 116: tiles.  400 of 56^2 39 and 23, 100 of 128^2 38 and 34, 200 of
+// 100^2 62 and 37: rows.  Estimates up to 5 % above go to the rows too (their
+// errors there: 128^2 takes 10 % less on them in either storage), and one
+// FP32 lattice up to 15 % above (61 x 21001: 32 us on either).
+inline bool rows_pay(const std::vector<LatDev>& lats, int height, bool f16, bool mrt, bool one,
+                     bool tensor, int64_t sms) {
+    return rows_us(lats, height, f16, mrt, one, sms) <
+           (one && !f16 ? 1.15 : 1.05) * tiles_us(lats, mrt, tensor);
+}
+
 // 32-bit offsets of k_rows2: a lattice's rows in a plane take less than 4 GB
 inline bool rows_fit(const LatDev& L, int es) {
     return ((int64_t)L.ny + 2 * GY) * L.pitch * es < (int64_t)1 << 32;

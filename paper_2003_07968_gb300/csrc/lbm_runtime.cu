@@ -158,6 +158,7 @@ struct lbm_handle {
     // row items of the lattices for the row kernel of their storage (none: no plan)
     int4* items = nullptr;
     int n_items = 0;
+    int item_rows = 0;  // of the tallest
     size_t items_bytes = 0;
     StepPath path = PATH_TILES;
     // the lattices as resident tiles, when they fit (plan_resident): tiles,
@@ -383,6 +384,7 @@ int make_items(lbm_handle* h) {
     h->items = (int4*)dev_alloc(h, h->items_bytes);
     if (!h->items) return LBM_ERR_OOM;
     h->n_items = (int)t.size();
+    h->item_rows = height;
     h->sent.push_back(std::move(t));
     CK(h, cudaMemcpyAsync(h->items, h->sent.back().data(), h->items_bytes, cudaMemcpyHostToDevice,
                           h->stream));
@@ -1109,15 +1111,18 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         const int rc = make_resident(h);
         if (rc) return fail(rc);
     }
-    // ... and larger ones run on the row kernels
+    // ... and larger ones run on the row kernels where their strips are filled
     if (!h->res_grid && fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
         !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
         const int rc = make_items(h);
         if (rc) return fail(rc);
         h->path = !h->items ? PATH_TILES
                   : tuned   ? tuned_path
-                  : h->f16  ? PATH_ROWS
-                            : PATH_PAIRS;  // measured: see k_rows2
+                  : !rows_pay(h->lat, h->item_rows, h->f16, h->collision == LBM_COLL_MRT, n == 1,
+                              cfg[1].variant == LBM_KERNEL_TMA, h->sm_count)
+                      ? PATH_TILES
+                  : h->f16 ? PATH_ROWS
+                           : PATH_PAIRS;
     }
     h->tune_variant = variant;
     h->rec[0].name = "psi_pass";

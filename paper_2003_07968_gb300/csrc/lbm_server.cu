@@ -149,6 +149,9 @@ struct TableSet {
     size_t cap[2] = {0, 0};
     int ntiles[2] = {0, 0};
     int npair = 0;  // pair items after the ntiles[1] row items (0: single steps only)
+    // the chunk runs on the row kernels (heights of their items), else on tiles
+    bool rows = false;
+    int row_h = 0, pair_h = 0;
     std::vector<int> begin[2], count[2];
     // tickets of the lattices (in table order) that the lattice table and
     // tile lists describe; a chunk over the same lattices only rewrites the
@@ -187,7 +190,7 @@ struct lbm_server {
     float* psi_arena = nullptr;
     int64_t pitch = 0, plane = 0, row_cap = 0;  // of the row space (elements, rows)
     size_t pop_bytes = 0, psi_region = 0;
-    bool rows = false;     // single pass on the row kernels (tile lists are row items)
+    bool rows = false;     // chunks may run on the row kernels (their lists are row items)
     bool pairs = false;    // ... two steps a launch (FP32 storage)
     bool tma = false;      // single pass on the TMA kernel (one tensor map for the arena)
     CUtensorMap tmap[2]{};  // loads, stores
@@ -294,11 +297,12 @@ int pass_grid(lbm_server* S, int k, int ntiles) {
     return std::max(1, std::min(ntiles, S->sm_count * occ));
 }
 
-cudaError_t launch(lbm_server* S, int k, const StepArgs& a, int grid, cudaStream_t st) {
+cudaError_t launch(lbm_server* S, int k, const StepArgs& a, int grid, cudaStream_t st,
+                   bool rows = false) {
     const PassState& P = S->pass[k];
     const dim3 block(P.tx, P.ty / P.spt);
     if (k == 0) return launch_psi(S->f16, S->o.eos_precision, P.spt, a, dim3(grid), block, st);
-    if (S->rows) return launch_rows(S->f16, 0, a, nullptr, st);
+    if (rows) return launch_rows(S->f16, 0, a, nullptr, st);
     if (S->tma)
         return launch_fused_tma(S->f16, 0, S->o.eos_precision, P.tx, P.ty, a, S->tmap, nullptr,
                                 grid, st);
@@ -322,13 +326,29 @@ StepArgs args(lbm_server* S, const TableSet& T, int k, int parity) {
     return a;
 }
 
+std::vector<uint64_t> tickets_of(const std::vector<Request*>& res) {
+    std::vector<uint64_t> t(res.size());
+    for (size_t i = 0; i < res.size(); ++i) t[i] = res[i]->ticket;
+    return t;
+}
+
+// Whether the resident requests run on the row kernels, and their items'
+// heights (the same lattices in the same order: as the set has it).
+void choose_rows(lbm_server* S, TableSet& T, const std::vector<Request*>& res) {
+    if (!S->rows || tickets_of(res) == T.members) return;
+    std::vector<LatDev> lats;
+    for (const Request* R : res) lats.push_back(R->L);
+    T.row_h = row_item_height(lats, (int64_t)S->sm_count * 4 * kRowWarps);
+    T.pair_h = S->pairs ? pair_item_height(lats, (int64_t)S->sm_count * 2 * kPairs) : 0;
+    T.rows = rows_pay(lats, S->pairs ? T.pair_h : T.row_h, S->f16, false, false, true, S->sm_count);
+}
+
 // Fill table set T from the resident requests with their chunk quotas,
 // through its pinned mirrors (the caller has waited for the set's previous
 // chunk, so the mirrors' last uploads are done).
 cudaError_t rebuild(lbm_server* S, TableSet& T, std::vector<Request*>& res,
                     const std::vector<int>& quota) {
-    std::vector<uint64_t> members(res.size());
-    for (size_t i = 0; i < res.size(); ++i) members[i] = res[i]->ticket;
+    std::vector<uint64_t> members = tickets_of(res);
     cudaError_t e = cudaSuccess;
     if (!res.empty()) {
         std::memcpy(T.quota_h, quota.data(), quota.size() * sizeof(int));
@@ -350,19 +370,14 @@ cudaError_t rebuild(lbm_server* S, TableSet& T, std::vector<Request*>& res,
     if (e != cudaSuccess) return e;
     for (int k = 0; k < 2; ++k) {
         const PassState& P = S->pass[k];
-        const bool items = k == 1 && S->rows;
+        const bool items = k == 1 && T.rows;
         size_t nt = 0, nrow = 0;
         std::vector<int4> rt;
         if (items) {
-            std::vector<LatDev> lats;
-            for (Request* R : res) lats.push_back(R->L);
-            const int height = row_item_height(lats, (int64_t)S->sm_count * 4 * kRowWarps);
-            for (size_t l = 0; l < res.size(); ++l) row_items(lats[l], (int)l, height, rt);
+            for (size_t l = 0; l < res.size(); ++l) row_items(res[l]->L, (int)l, T.row_h, rt);
             nrow = rt.size();
-            if (S->pairs) {
-                const int h2 = pair_item_height(lats, (int64_t)S->sm_count * 2 * kPairs);
-                for (size_t l = 0; l < res.size(); ++l) row_items(lats[l], (int)l, h2, rt, kPairCols);
-            }
+            for (size_t l = 0; l < res.size() && S->pairs; ++l)
+                row_items(res[l]->L, (int)l, T.pair_h, rt, kPairCols);
             nt = rt.size();
             T.npair = (int)(nt - nrow);
         }
@@ -666,6 +681,9 @@ void worker_loop(lbm_server* S) {
             C.res = res;
             C.p0 = S->parity;
             C.quota.resize(res.size());
+            TableSet& T = S->set[cur];
+            choose_rows(S, T, res);
+            const bool pairs = T.rows && S->pairs;
             // steps of this chunk: about chunk_ms of GPU time over the
             // resident sites, at most chunk_steps; an even number where two
             // steps go in a launch, so that lattices that run on end together
@@ -677,7 +695,7 @@ void worker_loop(lbm_server* S) {
                 const double fit = S->o.chunk_ms * 1e-3 * rate / (double)std::max<int64_t>(res_sites, 1);
                 steps = std::max<int64_t>(1, std::min<int64_t>(steps, (int64_t)fit));
             }
-            if (S->pairs) steps = std::max<int64_t>(2, steps & ~(int64_t)1);
+            if (pairs) steps = std::max<int64_t>(2, steps & ~(int64_t)1);
             int64_t k = 0;
             std::vector<Request*> keep;
             for (size_t l = 0; l < res.size(); ++l) {
@@ -690,20 +708,19 @@ void worker_loop(lbm_server* S) {
                     // (a launch, of one step or two, swaps the buffers)
                     C.finished.push_back(
                         Finished{res[l], (int)l,
-                                 (C.p0 + (S->pairs ? (C.quota[l] + 1) / 2 : C.quota[l])) & 1, LBM_OK});
+                                 (C.p0 + (pairs ? (C.quota[l] + 1) / 2 : C.quota[l])) & 1, LBM_OK});
             }
-            TableSet& T = S->set[cur];
             if (e == cudaSuccess) e = rebuild(S, T, C.res, C.quota);
             if (e == cudaSuccess) e = cudaEventRecord(S->chunk_begin[cur], S->stream);
             const int g0 = pass_grid(S, 0, T.ntiles[0]), g1 = pass_grid(S, 1, T.ntiles[1]);
-            for (int64_t st = 0; S->pairs && st < k && e == cudaSuccess; st += 2) {
+            for (int64_t st = 0; pairs && st < k && e == cudaSuccess; st += 2) {
                 // two steps of every lattice with at least two left, one of
                 // those with one
                 StepArgs a1 = args(S, T, 1, S->parity);
                 a1.step = (int)st;
                 if (std::any_of(C.quota.begin(), C.quota.end(), [&](int q) { return q == st + 1; })) {
                     a1.last_only = 1;
-                    e = launch(S, 1, a1, g1, S->stream);
+                    e = launch(S, 1, a1, g1, S->stream, true);
                     a1.last_only = 0;
                     ++launches;
                 }
@@ -715,11 +732,11 @@ void worker_loop(lbm_server* S) {
                 }
                 S->parity ^= 1;
             }
-            for (int64_t st = 0; !S->pairs && st < k && e == cudaSuccess; ++st) {
+            for (int64_t st = 0; !pairs && st < k && e == cudaSuccess; ++st) {
                 StepArgs a0 = args(S, T, 0, S->parity), a1 = args(S, T, 1, S->parity);
                 a0.step = a1.step = (int)st;
                 if (!S->fused) e = launch(S, 0, a0, g0, S->stream);
-                if (e == cudaSuccess) e = launch(S, 1, a1, g1, S->stream);
+                if (e == cudaSuccess) e = launch(S, 1, a1, g1, S->stream, T.rows);
                 launches += S->fused ? 1 : 2;
                 S->parity ^= 1;
             }

@@ -138,6 +138,39 @@ def test_autotune_leaves_the_paths_it_did_not_time(P):
     P.lbm_destroy(h)
 
 
+# -------------------------------------------------------------- chosen kernels
+@pytest.mark.parametrize("storage", [1, 2])
+@pytest.mark.parametrize("n,nx,ny", [(310, 64, 64), (1000, 32, 32), (400, 60, 60), (400, 56, 56)])
+def test_batches_run_no_slower_than_on_the_tile_kernel(P, n, nx, ny, storage):
+    # strips of 64 columns that hold half as many: the row kernels took up to
+    # twice the tile kernel's time there.  A given grid keeps a handle on the
+    # tile kernel; bitwise the same, and no slower (8 % for noise)
+    import time
+
+    descs = [P.lbm_desc_default(nx, ny, T=0.8, storage=storage)] * n
+    fields = [_field(nx, ny, k % 5) for k in range(5)]
+    grid, best, out = 0, [], []
+    for kw in ({}, {"grid_ctas": 0}):
+        h = P.lbm_create(descs, **{k: grid for k in kw})
+        grid = P.lbm_info(h)["grid_ctas"]
+        for i in range(n):
+            P.lbm_init(h, i, fields[i % 5])
+        t = []
+        for _ in range(6):
+            P.lbm_sync(h)
+            t0 = time.perf_counter()
+            P.lbm_step(h, 128)
+            P.lbm_sync(h)
+            t.append(time.perf_counter() - t0)
+        best.append(min(t))
+        out.append([P.lbm_moments(h, i) for i in (0, 1, n - 1)])
+        P.lbm_destroy(h)
+    for a, b in zip(*out):
+        _same(a, b)
+    print(n, nx, ny, storage, [f"{t / 128e-6:.1f} us" for t in best])
+    assert best[0] <= 1.08 * best[1]
+
+
 # ------------------------------------------------------------------ records
 def test_profile_read_gives_at_most_max_records(P):
     import ctypes
