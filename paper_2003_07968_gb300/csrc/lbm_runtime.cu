@@ -476,6 +476,17 @@ int launch_resident_steps(lbm_handle* h, int nsteps) {
     return LBM_OK;
 }
 
+// While it lives, a capture that the caller has in progress on another stream
+// (of any thread, in global mode) neither forbids this thread's event queries
+// and creations nor is ended by them: none of them touches what it captures.
+struct BesideCaptures {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~BesideCaptures() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    BesideCaptures(const BesideCaptures&) = delete;
+    BesideCaptures& operator=(const BesideCaptures&) = delete;
+};
+
 cudaEvent_t take_event(lbm_handle* h) {
     if (!h->ev_pool.empty()) {
         cudaEvent_t e = h->ev_pool.back();
@@ -1199,6 +1210,7 @@ int lbm_init(lbm_handle* h, int32_t lattice, const double* rho, const double* ux
 
 static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     if (!h || nsteps < 0) return LBM_ERR_ARG;
+    const BesideCaptures beside;
     // Into a caller's stream capture goes one launch per step and nothing else:
     // a graph of the handle's own can be neither captured nor launched there, a
     // replayed resident launch would not be counted among those in flight, an

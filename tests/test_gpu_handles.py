@@ -115,6 +115,33 @@ def test_replays_alternate_with_direct_steps(P, shape, storage, kw):
         _same(got, _tile_run(P, d, f, steps + 7))
 
 
+def test_steps_beside_a_capture_of_another_stream(P):
+    # a capture in global mode (torch's default) forbids event queries to the
+    # whole process, and lbm_step of a handle on another stream asks how its
+    # resident launches and fault words stand: its steps still run at once, and
+    # the capture ends as if they had not been there
+    import torch
+
+    d, f = P.lbm_desc_default(64, 50, T=0.8), _field(64, 50)
+    other, h = P.lbm_create(d), P.lbm_create(d)
+    for x in (other, h):
+        P.lbm_init(x, 0, f)
+    P.lbm_step(other, 4)  # a resident launch in the list of those in flight
+    P.lbm_sync(other)
+    v, g = torch.zeros(8, device="cuda"), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        v += 1
+        P.lbm_step(h, 4)
+        P.lbm_step(h, 3)  # the first call's fault words are on their way
+    g.replay()
+    torch.cuda.synchronize()
+    assert v.eq(1).all()
+    got = P.lbm_moments(h, 0)
+    for x in (other, h):
+        P.lbm_destroy(x)
+    _same(got, _tile_run(P, d, f, 7))
+
+
 # ------------------------------------------------------------ tuned choices
 def test_autotune_leaves_the_paths_it_did_not_time(P):
     # two lattices tuned on a handle that has no row kernel (resident) and a
