@@ -205,20 +205,25 @@ struct ResArgs {
 // Bands of a lattice of ny rows when tiles of about `rows` rows are aimed at.
 inline int res_bands(int ny, int rows) { return std::max(1, std::min((ny + rows - 1) / rows, ny / 2)); }
 
+// Rows of the tiles that a launch takes beside others: with psi's two more they
+// are two rounds of the eight warps.
+constexpr int kResBeside = 14;
+
 struct ResPlan {
     std::vector<ResTile> tiles;  // none: no plan
     int rows = 0;  // of the tallest tile
 };
 
 // The tiles of a handle's lattices if each block of a launch of at most
-// `blocks` can keep one: the flattest tiles that fit.  Flat tiles spread the
-// rows over all SMs, and a step is latency: 256^2 takes 2.73 us a step in 260
-// tiles of 4 rows, 2.95 in 145 of 8 and 4.3 in 60 of 21.
-inline ResPlan plan_resident(const std::vector<LatDev>& lats, int blocks, int es) {
+// `blocks` can keep one: the flattest tiles (of about `low` rows or more) that
+// fit.  Flat tiles spread the rows over all SMs, and a step is latency: 256^2
+// takes 2.73 us a step in 260 tiles of 4 rows, 2.95 in 145 of 8 and 4.3 in 60
+// of 21.
+inline ResPlan plan_resident(const std::vector<LatDev>& lats, int blocks, int es, int low = 2) {
     ResPlan P;
     const int most = res_rows(es);
     int h = 0;  // the smallest height whose tiles fit
-    for (int rows = 2; rows <= most && !h; ++rows) {
+    for (int rows = low; rows <= most && !h; ++rows) {
         int64_t n = 0;
         int tallest = 0;
         for (const LatDev& L : lats) {

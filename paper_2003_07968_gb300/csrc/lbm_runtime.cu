@@ -48,6 +48,13 @@ struct TuneKey {
 struct PassCfg {
     int variant, tx, ty, grid, spt;
 };
+// Tiles that a handle's lattices are cut into for k_resident: their count (0: no
+// such cut), packets of a mailbox slot, and where tiles, mailboxes and epochs
+// lie in the handle's allocation.
+struct ResCut {
+    int grid = 0, slot = 0;
+    size_t tiles = 0, mail = 0, epoch = 0;
+};
 // What the single pass runs on: the tile kernels of pass[1], k_rows, or
 // k_rows2 (two steps a launch, an odd step on the tile kernel).
 enum StepPath { PATH_TILES, PATH_ROWS, PATH_PAIRS };
@@ -161,11 +168,11 @@ struct lbm_handle {
     int item_rows = 0;  // of the tallest
     size_t items_bytes = 0;
     StepPath path = PATH_TILES;
-    // the lattices as resident tiles, when they fit (plan_resident): tiles,
-    // mailboxes and epochs in one allocation
-    int res_grid = 0;  // tiles (0: no plan)
+    // the lattices as resident tiles, when they fit (plan_resident): the
+    // flattest tiles and, for launches beside other handles', fewer and taller
+    // ones, each with mailboxes and epochs of its own; in one allocation
+    ResCut cut[2];
     size_t res_bytes = 0;
-    int res_slot = 0;
     void* res = nullptr;
     bool res_reset = true;  // mailboxes and epochs must be cleared first
     // profiling
@@ -339,31 +346,43 @@ cudaError_t launch_pass(lbm_handle* h, int k, const StepArgs& a, int grid) {
                                 h->stream);
 }
 
-// Tiles, mailboxes and epochs of the handle's resident plan in h->res.
-ResTile* res_tiles(lbm_handle* h) { return static_cast<ResTile*>(h->res); }
-size_t res_mail_off(const lbm_handle* h) {
-    return (size_t)round_up((int64_t)(h->res_grid * sizeof(ResTile)), 256);
-}
-size_t res_epoch_off(const lbm_handle* h) {
-    return res_mail_off(h) + (size_t)h->res_grid * 2 * h->res_slot * sizeof(uint4);
-}
-
-// Plan the handle's lattices as resident tiles.  LBM_OK without a plan too.
+// Cut the handle's lattices into resident tiles.  LBM_OK without a cut too.
+//
+// The flattest tiles take a step in the least time but may take all SMs even for
+// a small lattice (128^2: 192 of the 304 blocks that fit), and launches of
+// other handles then run one after another.  Where half of the blocks or fewer
+// hold the lattices in tiles of kResBeside rows, launches beside others take
+// those, so that two and more go on at the same time.
 int make_resident(lbm_handle* h) {
     int coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, h->device) != cudaSuccess || !coop)
         return LBM_OK;
-    ResPlan P = plan_resident(h->lat, std::min(2 * h->sm_count, kResBlocks), h->f16 ? 2 : 4);
-    if (P.tiles.empty()) return LBM_OK;
+    const int es = h->f16 ? 2 : 4;
+    ResPlan P[2];
+    P[0] = plan_resident(h->lat, std::min(2 * h->sm_count, kResBlocks), es);
+    if (P[0].tiles.empty()) return LBM_OK;
     const int per_sm =
         resident_blocks_per_sm(h->f16, h->collision == LBM_COLL_MRT, h->lat.size() == 1);
     if (per_sm < 2) return LBM_OK;  // the flights are counted at two blocks an SM
-    h->res_grid = (int)P.tiles.size();
-    h->res_slot = res_packets(P.rows, kRowCols);
-    h->res_bytes = res_epoch_off(h) + h->res_grid * sizeof(uint32_t);
+    if (P[0].rows < kResBeside) {
+        P[1] = plan_resident(h->lat, std::min(h->sm_count, (int)P[0].tiles.size() - 1), es, kResBeside);
+        if (P[1].rows > kResBeside) P[1].tiles.clear();
+    }
+    size_t at = (P[0].tiles.size() + P[1].tiles.size()) * sizeof(ResTile);
+    for (int k = 0; k < 2; ++k) {
+        ResCut& C = h->cut[k];
+        C.grid = (int)P[k].tiles.size();
+        C.slot = res_packets(P[k].rows, kRowCols);
+        C.tiles = k ? P[0].tiles.size() * sizeof(ResTile) : 0;
+        C.mail = at = (size_t)round_up((int64_t)at, 256);
+        C.epoch = at += (size_t)C.grid * 2 * C.slot * sizeof(uint4);
+        at += C.grid * sizeof(uint32_t);
+    }
+    h->res_bytes = at;
     h->res = dev_alloc(h, h->res_bytes);
     if (!h->res) return LBM_ERR_OOM;
-    h->sent_tiles = std::move(P.tiles);
+    h->sent_tiles = std::move(P[0].tiles);
+    h->sent_tiles.insert(h->sent_tiles.end(), P[1].tiles.begin(), P[1].tiles.end());
     CK(h, cudaMemcpyAsync(h->res, h->sent_tiles.data(), h->sent_tiles.size() * sizeof(ResTile),
                           cudaMemcpyHostToDevice, h->stream));
     return LBM_OK;
@@ -404,31 +423,18 @@ cudaError_t launch_row_steps(lbm_handle* h, int parity, int32_t starve = 0) {
 }
 
 // nsteps steps in one launch (state from buffer `parity` to the other).
-// LBM_PENDING (nothing launched, no plan any more) where the device grants
-// this process fewer SMs than the plan needs.
+// LBM_PENDING (nothing launched, no cuts any more) where the device grants
+// this process fewer SMs than the launch needs.
 int launch_resident_steps(lbm_handle* h, int nsteps) {
+    char* const base = static_cast<char*>(h->res);
     if (h->res_reset) {
-        CK(h, cudaMemsetAsync(static_cast<char*>(h->res) + res_mail_off(h), 0,
-                              h->res_bytes - res_mail_off(h), h->stream));
+        CK(h, cudaMemsetAsync(base + h->cut[0].mail, 0, h->res_bytes - h->cut[0].mail, h->stream));
         h->res_reset = false;
-    }
-    ResArgs m{};
-    m.a = step_args(h, h->parity, 1);
-    m.tiles = res_tiles(h);
-    m.mail = reinterpret_cast<uint4*>(static_cast<char*>(h->res) + res_mail_off(h));
-    m.epoch = reinterpret_cast<uint32_t*>(static_cast<char*>(h->res) + res_epoch_off(h));
-    m.slot = h->res_slot;
-    m.nsteps = nsteps;
-    if (h->starve_item) {
-        // an armed failure-detection test: the tile's packets carry numbers that
-        // none of its neighbours waits for (lbm_init clears the epochs)
-        CK(h, cudaMemsetAsync(m.epoch + (h->starve_item - 1), 0x80, sizeof(uint32_t), h->stream));
-        m.a.wait_cycles = kTestWaitBudgetCycles;
-        h->starve_item = 0;
     }
     Flights& F = flights_of(h->device);
     std::lock_guard<std::mutex> lk(F.mu);
     auto mine = F.list.end();
+    int others = 0;  // blocks of the other streams' launches
     for (auto it = F.list.begin(); it != F.list.end();) {
         const cudaError_t q = cudaEventQuery(it->done);
         if (q == cudaSuccess) {
@@ -437,11 +443,38 @@ int launch_resident_steps(lbm_handle* h, int nsteps) {
             continue;
         }
         if (q != cudaErrorNotReady) return cuda_fail(h, q, "cudaEventQuery");
-        if (it->stream == h->stream) mine = it;
+        if (it->stream == h->stream)
+            mine = it;
+        else
+            others += it->blocks;
         ++it;
     }
+    // The tall tiles where the flat ones do not fit beside all others.  Handles of
+    // one lattice on streams of their own, 512 steps a call, us a step of all on
+    // flat tiles only -> so (on the tile kernel):
+    //   4, 8, 32 of 128^2   8.7, 17.5, 70.1 -> 3.6, 6.7, 16.0    (6.2, 7.3, 27.9)
+    //   4, 8, 32 of 256^2  10.9, 21.8, 87.4 -> 7.2, 14.3, 46.9   (8.1, 15.7, 63.3)
+    // Few may wait for one another either way, then in more time: 2 of 256^2 5.5 ->
+    // 6.0 (6.7), 4 of 100^2 4.3 -> 5.4 (6.2).  An armed failure-detection test is
+    // for the flat tiles.
+    const int slots = 2 * h->sm_count;
+    const ResCut& C = h->cut[others + h->cut[0].grid > slots && h->cut[1].grid && !h->starve_item];
+    ResArgs m{};
+    m.a = step_args(h, h->parity, 1);
+    m.tiles = reinterpret_cast<ResTile*>(base + C.tiles);
+    m.mail = reinterpret_cast<uint4*>(base + C.mail);
+    m.epoch = reinterpret_cast<uint32_t*>(base + C.epoch);
+    m.slot = C.slot;
+    m.nsteps = nsteps;
+    if (h->starve_item) {
+        // an armed failure-detection test: the tile's packets carry numbers that
+        // none of its neighbours waits for (lbm_init clears the epochs)
+        CK(h, cudaMemsetAsync(m.epoch + (h->starve_item - 1), 0x80, sizeof(uint32_t), h->stream));
+        m.a.wait_cycles = kTestWaitBudgetCycles;
+        h->starve_item = 0;
+    }
     // beside which of the other streams' launches it fits, the newest first
-    int room = 2 * h->sm_count - h->res_grid;
+    int room = slots - C.grid;
     bool fits = true;
     for (auto it = F.list.rbegin(); it != F.list.rend(); ++it) {
         if (it->stream == h->stream) continue;
@@ -460,13 +493,13 @@ int launch_resident_steps(lbm_handle* h, int nsteps) {
     }
     const cudaError_t e =
         launch_resident(h->f16, h->collision == LBM_COLL_MRT, m,
-                        h->lat.size() == 1 ? &h->lat[0] : nullptr, h->res_grid, h->stream);
-    if (e == cudaSuccess) mine->blocks = std::max(mine->blocks, h->res_grid);
+                        h->lat.size() == 1 ? &h->lat[0] : nullptr, C.grid, h->stream);
+    if (e == cudaSuccess) mine->blocks = std::max(mine->blocks, C.grid);
     // (a record after a failed launch only marks the work queued before it)
     const cudaError_t r = cudaEventRecord(mine->done, h->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {
         cudaGetLastError();
-        h->res_grid = 0;
+        h->cut[0].grid = 0;
         return r == cudaSuccess ? LBM_PENDING : cuda_fail(h, r, "cudaEventRecord");
     }
     if (e != cudaSuccess) return cuda_fail(h, e, "resident launch");
@@ -1123,7 +1156,7 @@ static int lbm_create_body(const lbm_lattice_desc* descs, int32_t n, const lbm_r
         if (rc) return fail(rc);
     }
     // ... and larger ones run on the row kernels where their strips are filled
-    if (!h->res_grid && fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
+    if (!h->cut[0].grid && fused && variant == LBM_KERNEL_AUTO && h->eos == LBM_EOS_DF &&
         !(opts && (opts->tile_x || opts->tile_y || opts->grid_ctas))) {
         const int rc = make_items(h);
         if (rc) return fail(rc);
@@ -1225,7 +1258,7 @@ static int lbm_step_body(lbm_handle* h, int64_t nsteps) {
     // resident lattices: from two steps on (one step is one tile-kernel launch;
     // a resident one costs about 3 us beside its steps).  A launch swaps the
     // buffers once, so a captured handle's launches take odd numbers of steps.
-    if (direct && h->res_grid && !h->prof && !h->starve) {
+    if (direct && h->cut[0].grid && !h->prof && !h->starve) {
         while (left >= (h->captured ? 3 : 2)) {
             // at most 2^14 steps a launch (a fraction of a second)
             int n = (int)std::min<int64_t>(left, left == (1 << 14) + 1 ? 1 << 13 : 1 << 14);
@@ -1602,7 +1635,7 @@ int lbm_inject_copy_timeout(lbm_handle* h, int32_t tile) {
 
 static int lbm_inject_wait_timeout_body(lbm_handle* h, int32_t item) {
     if (!h) return LBM_ERR_ARG;
-    const int n = h->res_grid ? h->res_grid : h->path == PATH_PAIRS ? h->n_items : 0;
+    const int n = h->cut[0].grid ? h->cut[0].grid : h->path == PATH_PAIRS ? h->n_items : 0;
     if (item < 0 || item >= n) return LBM_ERR_ARG;
     h->starve_item = item + 1;  // the next launch of many or of two steps; no graph replays it
     return LBM_OK;
