@@ -185,13 +185,13 @@ __device__ __forceinline__ int item_width(int w) { return w >> 24; }
 // h + 2 and reads h + 4; a tile kernel's 32 x 16 tile computes it for 18 x 34
 // sites, fetches 20 x 40 and holds its warps at a barrier per tile.
 //
-// What bounds it: FP16 storage the FP32 pipe (75 % of its cycles; 61 % of
-// issue slots; paired instructions take two cycles), FP32 storage beyond L2
-// DRAM.  Measured per step, tile kernel (32 x 16) -> this one:
-//   FP16       4096^2 244 -> 190 us, 8192^2 937 -> 688 us (97.6 GLUPS);
-//              MRT 288 -> 230 and 1112 -> 846 us
-//   FP32 BGK   900^2 16.5 -> 14.9, 1200^2 33.4 -> 22.8; 4096^2 222 -> 235
-//              (there it takes the odd step beside k_rows2 only)
+// What bounds it: FP16 storage the FP32 pipe (its heavy half is busy 73 % of its
+// cycles, 64 % of issue slots; paired instructions take two cycles), FP32
+// storage beyond L2 DRAM.  Measured per step, tile kernel (32 x 16) -> this one,
+// FP16: 4096^2 244 -> 190 us, 8192^2 937 -> 688 us (97.6 GLUPS); MRT 288 -> 230
+// and 1112 -> 846 us.  FP32 storage has the batch instance only, for the last
+// step of served requests with an odd number of steps (k_rows2 takes the others;
+// on handles the tile kernel takes an odd step); it spills 76 bytes.
 // Unrolling the row loop by 2 to save its register copies gained 4 % in FP16
 // BGK and spilled in the others (MRT 10 % slower); 5 blocks an SM spill too.
 template <class S, int EOSP, bool MRT, bool ONE>
@@ -263,20 +263,10 @@ __global__ void __launch_bounds__(32 * kRowWarps, 4)
 }
 
 // ---------------------------------------------------------------- two steps a launch
-// A pair's raw value from two columns of a row.
-__device__ __forceinline__ float2 raw_of(float a, float b) { return make_float2(a, b); }
-__device__ __forceinline__ uint32_t raw_of(__half a, __half b) {
-    return (uint32_t)__half_as_ushort(a) | (uint32_t)__half_as_ushort(b) << 16;
-}
 __device__ __forceinline__ float ld_one(const float* p) {
     float v;
     asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
-}
-__device__ __forceinline__ __half ld_one(const __half* p) {
-    unsigned short v;
-    asm volatile("ld.global.cg.b16 %0, [%1];" : "=h"(v) : "l"(p));
-    return __ushort_as_half(v);
 }
 
 // k_rows2: two steps; a pair of warps marches down an item's rows.  The first
@@ -288,7 +278,9 @@ __device__ __forceinline__ __half ld_one(const __half* p) {
 //
 // One step a launch moves 72 bytes a site and step (FP32) and stops at 0.81 of
 // the copy bandwidth; two move 36, and the kernel is bound by the FP32 pipe
-// (73 % of its cycles, 63 % of issue slots).  Measured per step, 32 x 16 tile
+// (72 % of its heavy half's cycles, 63 % of issue slots).  The batch instances
+// hold the lattice's constants in registers beside the rows and spill (100
+// bytes, MRT 28); the others do not.  Measured per step, 32 x 16 tile
 // kernel -> this one: FP32 BGK 1024^2 19.2 -> 16.3 us, 1201^2 33.2 -> 21.6,
 // 2100 x 1700 51.6 -> 46.2, 4096^2 221 -> 191, 8192^2 870 -> 706 (95 GLUPS);
 // MRT 8192^2 984 -> 865; 512 lattices of 64^2 .. 512^2 804 -> 730, 100 of
@@ -296,12 +288,13 @@ __device__ __forceinline__ __half ld_one(const __half* p) {
 // the columns it computes twice (8192^2: k_rows 688, this one 778).
 // Unrolling either row loop by 2 is 3 to 25 % slower; 64-bit addresses and a
 // test per load instead of one per row cost 6 %.
-template <class S, int EOSP, bool MRT, bool ONE>
+template <int EOSP, bool MRT, bool ONE>
 __global__ void __launch_bounds__(64 * kPairs, 2)
     k_rows2(StepArgs a, const __grid_constant__ LatDev lat0) {
-    using T = typename S::T;
+    using S = StoreF32;
+    using T = S::T;
     using IO = PairIO<S>;
-    using Raw = typename IO::Raw;
+    using Raw = IO::Raw;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ LatDev slat[ONE ? 1 : kPairs];
     __shared__ uint64_t bars[kPairs][2 * kPairDepth];
@@ -359,7 +352,7 @@ __global__ void __launch_bounds__(64 * kPairs, 2)
             return reinterpret_cast<const T*>(base + i * plane * (int64_t)sizeof(T) + o);
         };
         auto one = [&](int i, uint32_t o) {
-            return raw_of(ld_one(at(i, o)), ld_one(at(i, o + (uint32_t)next)));
+            return make_float2(ld_one(at(i, o)), ld_one(at(i, o + (uint32_t)next)));
         };
         auto ld = [&](int i, uint32_t o) { return whole ? IO::ld(at(i, o)) : one(i, o); };
         auto load = [&](Raw g[9], Raw& rest, uint32_t om, uint32_t oc, uint32_t op) {
@@ -529,14 +522,14 @@ __device__ __forceinline__ int halo_line(int k) { return k < 4 ? 0 : k < 10 ? 1 
 //
 // What bounds it: latency.  A launch per step costs 5.2-5.4 us for any
 // lattice up to about 256^2 (launch, first loads, psi barrier, stores and the
-// end of the grid, one after another); here a step is psi (about 1000
-// cycles), collision (1000-1500), and the exchange (packets out 1000 cycles,
-// and in 2300: two trips to L2).  Measured per step, FP32, one launch per
-// step in a graph -> here: 64^2 5.2 -> 2.0 us, 200^2 MRT 5.4 -> 2.5 us, 256^2
-// 5.3 -> 2.7 us, 777 x 611 11.0 -> 7.2 us.  Flags behind release fences
-// instead of tagged packets took 3.0 us at 64^2 and 5.3 us at 256^2 (the
-// fence alone waits 2200 cycles for the stores before it); 8-byte packets of
-// one value 2.1 and 3.2 us.
+// end of the grid, one after another); here a step is psi and collision (950
+// cycles at 64^2, 1450 at 256^2, 8800 for the 21 rows a tile of 777 x 611),
+// packets out (1050, 1400, 1300) and packets in (2000, 2550, 4500 with the wait
+// for the slowest neighbour): two trips to L2.  Measured per step, FP32, one
+// launch per step in a graph -> here: 64^2 5.2 -> 2.0 us, 200^2 MRT 5.4 -> 2.5
+// us, 256^2 5.3 -> 2.7 us, 777 x 611 11.0 -> 7.2 us.  Flags behind release
+// fences instead of tagged packets took 3.0 us at 64^2 and 5.3 us at 256^2;
+// 8-byte packets of one value 2.1 and 3.2 us.
 //
 // Rows j = 0 .. rows + 1 of a tile's psi are lattice rows y0 - 1 .. y0 + rows.
 // A round is eight rows, one a warp: pulled state and psi of the round's
@@ -779,27 +772,20 @@ cudaError_t rows_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-template <class S, bool MRT, bool ONE>
+template <bool MRT, bool ONE>
 cudaError_t pairs_inst(const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
-    constexpr int smem = (int)pair_smem((int)sizeof(typename S::T));
-    const cudaError_t e = cudaFuncSetAttribute((const void*)k_rows2<S, EOS_DF, MRT, ONE>,
+    constexpr int smem = (int)kPairSmem;
+    const cudaError_t e = cudaFuncSetAttribute((const void*)k_rows2<EOS_DF, MRT, ONE>,
                                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const unsigned grid = (unsigned)((a.ntiles + kPairs - 1) / kPairs);
-    k_rows2<S, EOS_DF, MRT, ONE><<<grid, 64 * kPairs, smem, st>>>(a, lat0 ? *lat0 : LatDev{});
+    k_rows2<EOS_DF, MRT, ONE><<<grid, 64 * kPairs, smem, st>>>(a, lat0 ? *lat0 : LatDev{});
     return cudaGetLastError();
 }
 
 }  // namespace
 
-// (FP32 storage only, see k_rows2)
-template <class S>
-cudaError_t pairs_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
-    if (mrt) return lat0 ? pairs_inst<S, true, true>(a, lat0, st) : pairs_inst<S, true, false>(a, lat0, st);
-    return lat0 ? pairs_inst<S, false, true>(a, lat0, st) : pairs_inst<S, false, false>(a, lat0, st);
-}
-
-// (FP32 storage: the odd steps of a server's requests only)
+// (FP32 storage: the odd last steps of a server's requests only)
 template <class S>
 cudaError_t rows_any(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
     if constexpr (sizeof(typename S::T) == 4)

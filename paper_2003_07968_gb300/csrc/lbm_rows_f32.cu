@@ -13,7 +13,8 @@ cudaError_t rows_f32(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_
 }
 
 cudaError_t pairs_f32(int mrt, const StepArgs& a, const LatDev* lat0, cudaStream_t st) {
-    return pairs_any<StoreF32>(mrt, a, lat0, st);
+    if (mrt) return lat0 ? pairs_inst<true, true>(a, lat0, st) : pairs_inst<true, false>(a, lat0, st);
+    return lat0 ? pairs_inst<false, true>(a, lat0, st) : pairs_inst<false, false>(a, lat0, st);
 }
 
 }  // namespace pplbm

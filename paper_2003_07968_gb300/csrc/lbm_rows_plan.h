@@ -10,9 +10,8 @@ namespace pplbm {
 
 constexpr int kRowCols = 60;  // columns a warp advances at most (it holds 64)
 
-// Column c of boundary k of n strips over nx columns: even, at most kRowCols
-// apart, as equal as that allows.
-// (n strips of at most `cols` columns each: strip_count)
+// First column of strip k of the n = strip_count(nx, cols) strips over nx columns:
+// even, two of them at most `cols` (an even number) apart, as equal as that allows.
 inline int strip_edge(int nx, int n, int k) {
     const int pairs = (nx + 1) / 2;
     return std::min(nx, 2 * (int)(((int64_t)pairs * k + n - 1) / n));
@@ -56,7 +55,7 @@ inline void row_items(const LatDev& L, int lattice, int h, std::vector<int4>& ou
 constexpr int kPairCols = 56;   // columns of an item at most (64 held, 4 lost a side)
 constexpr int kPairDepth = 8;   // rows of the ring between a pair's warps
 constexpr int kPairs = 4;       // pairs of a block
-constexpr size_t pair_smem(int es) { return (size_t)kPairs * kPairDepth * 9 * 64 * es; }
+constexpr size_t kPairSmem = (size_t)kPairs * kPairDepth * 9 * 64 * sizeof(float);
 
 // Rows of an item, `pairs`: the pairs of warps the GPU holds.  One wave while
 // that makes items of about 100 rows at most, then even waves of about 72
