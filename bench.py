@@ -3,8 +3,9 @@
 Default workload: one 8192 x 8192 FP32 droplet lattice (R = 2048, T_r = 0.8,
 BGK tau = 1, eps = 1.73, sigma = 1), the roofline configuration.  A "step"
 is one time step of the whole hot path over that lattice: pull, density,
-psi, force, collision and store, by default two steps in one kernel launch.  The working set (two population buffers, 4.8 GB) is far
-larger than L2, so no flush is needed between steps.
+psi, force, collision and store, by default two steps in one kernel launch.
+The working set (two population buffers, 4.8 GB) is far larger than L2, so no
+flush is needed between steps.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl gb300|reference]
                   [--workload roofline|batched|served]
@@ -39,6 +40,16 @@ sys.path.insert(0, ROOT)
 METRIC = ("MLUPS and % of HBM peak per step; batched/served p50/p99 vs plain FP32 at "
                    "1e-5")
 FALLBACK_HBM_GBS = 6800.0
+
+
+def bound(kernel, storage, eos):
+    """What the step's kernel runs into: the row kernels (two steps a launch, or
+    one in FP16 storage) the FP32 pipe (profiles/row_kernels_droplet4096.md), a
+    native FP64 EOS the FP64 pipe, else memory."""
+    if eos == "f64":
+        return "fp64"
+    rows = kernel == "fused_two_steps" or (kernel == "fused_step" and storage == "f16dev")
+    return "fp32" if rows else "hbm"
 
 
 def parse():
@@ -428,7 +439,9 @@ def run_gpu(args):
                    "l2": f"working set {info['device_bytes'] / 1e9:.2f} GB vs 129 MB L2: "
                          "inputs larger than L2, no flush",
                    "parallelism": f"replicas x{world}"},
-        "roofline": {"bound": "hbm", "kernel": dom["name"], "achieved": round(achieved, 1),
+        # (achieved, peak and frac are of HBM, whatever the kernel runs into)
+        "roofline": {"bound": bound(dom["name"], args.storage, args.eos), "kernel": dom["name"],
+                     "achieved": round(achieved, 1),
                      "peak": peak, "unit": "GB/s", "frac": round(achieved / peak, 4),
                      # a launch of two steps moves the same bytes as one of one
                      "steps_per_launch": 2 if dom["name"] == "fused_two_steps" else 1,
@@ -621,7 +634,8 @@ def run_batched(args):
                                        info["spt"], info["grid_ctas"]],
                       "schedule": ["auto", "two_pass", "fused"][info["schedule"]]},
            "batched": b,
-           "roofline": {"bound": "hbm", "kernel": b["kernel"]["name"],
+           "roofline": {"bound": bound(b["kernel"]["name"], args.storage, args.eos),
+                        "kernel": b["kernel"]["name"],
                         "achieved": b["kernel"]["achieved_GBps"], "peak": peak, "unit": "GB/s",
                         "frac": b["kernel"]["frac"], "traffic": None, "peak_source": peak_src},
            "gpu_launches": b["gpu_launches"], "clocks": b["clocks"]}
